@@ -23,7 +23,7 @@
 #include "solve_internal.h"
 #include "xinv_tma.cuh"
 #include "ypass_tma.cuh"
-#include "zsolve.cuh"
+#include "zcirc.cuh"
 
 namespace vofp {
 
@@ -45,6 +45,7 @@ static void allow_all() {
   allow_smem(xinv_kernel<T, C>());
   allow_smem(k_zsolve<T, T>);
   allow_smem(k_ztab<T, TT>);
+  allow_smem(k_zcirc<T>);
   allow_smem(k_ztab_staged<T, TT>);
   allow_smem(k_ztab_seg<T, TT, false>);
   allow_smem(k_ztab_seg<T, TT, true>);
@@ -361,6 +362,15 @@ static void solve_red(vofp_plan* pl, cudaStream_t st, int skip_k, double tol2, b
     if (pl->nlow > 0)
       VOFP_LAUNCH(KID_ZLOW, st,
                   k_zlow_scan<R><<<(pl->nlow + 3) / 4, 128, 0, st>>>(za, pl->lowmodes, pl->nlow, pl->lowtab,
+                                                                     pl->lowscratch));
+  } else if (pl->zcirc) {
+    const ZCircArgs zc = zcirc_args(pl);
+    const dim3 tgrid((nx + zc.ti - 1) / zc.ti, ny);
+    VOFP_LAUNCH(KID_ZSOLVE, st, (k_zcirc<R><<<tgrid, kZCircThreads, zcirc_smem(nz, zc.ti, sizeof(R)), st>>>(za, zc)));
+    if (pl->nlow > 0)
+      VOFP_LAUNCH(KID_ZLOW, st,
+                  k_zcirc_low<R><<<(pl->nlow + 3) / 4, 128, 0, st>>>(za, pl->lowmodes, pl->nlow,
+                                                                     (const ZCirc<double>*)pl->zcirc_low,
                                                                      pl->lowscratch));
   } else {
     const int nvec = pl->bc[2] == VOFP_BC_P ? 3 : 2;

@@ -20,7 +20,7 @@
 #include <vector>
 
 #include "solve_internal.h"
-#include "zsolve.cuh"
+#include "zcirc.cuh"
 #include "vofp_internal.cuh"
 
 namespace vofp {
@@ -417,6 +417,21 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     L.T = off;
     off = align256(off + tsz * (size_t)Ux * Uy * nz);
   }
+  // periodic z with equal widths: the circulant systems' factors
+  L.zcirc = L.zcirc_low = 0;
+  bool zuniform = zper && nz >= 3;
+  for (int k = 1; k < nz; ++k) zuniform = zuniform && dz[k] == dz[0];
+  if (zuniform) {
+    const size_t elem = mixed ? rs : sizeof(double);
+    p->zcirc_ti = zcirc_ti(nz, elem);
+    p->zcirc_rows = zcirc_rows(nz, p->zcirc_ti);
+    L.zcirc = off;
+    off = align256(off + 5 * elem * (size_t)Ux * Uy);
+    if (!low.empty()) {
+      L.zcirc_low = off;
+      off = align256(off + sizeof(ZCirc<double>) * low.size());
+    }
+  }
   // FP32 refinement plans: the x transform matrices of the tensor-core x passes
   L.xtc = 0;
   const size_t xb = xtc_table_bytes(nx, (long)ny * nz, o.prec);
@@ -594,6 +609,12 @@ int plan_bind(PlanPrep* pp, void* block, cudaStream_t st, unsigned char* stage) 
   init_kernel_attributes_mixed();
   if (p->ztab) {
     const int s = build_z_factors(p, st, own);
+    if (s) return s;
+  }
+  p->zcirc = L.zcirc ? (void*)(b + L.zcirc) : nullptr;
+  p->zcirc_low = L.zcirc_low ? (void*)(b + L.zcirc_low) : nullptr;
+  if (p->zcirc) {
+    const int s = build_zcirc(p, st, own);
     if (s) return s;
   }
   if (p->lowtab) {

@@ -12,7 +12,7 @@
 #include "epilogue.cuh"
 #include "passes.cuh"
 #include "solve_internal.h"
-#include "zsolve.cuh"
+#include "zcirc.cuh"
 
 using namespace vofp;
 
@@ -75,6 +75,7 @@ void init_kernel_attributes_fp64() {
   allow_smem(k_xinv_f64<0>);
   allow_smem(k_zsolve<double, double>);
   allow_smem(k_ztab<double, ZF<double>>);
+  allow_smem(k_zcirc<double>);
   allow_smem(k_ztab_staged<double, ZF<double>>);
   allow_smem(k_ztab_seg<double, ZF<double>, false>);
   allow_smem(k_ztab_seg<double, ZF<double>, true>);
@@ -123,6 +124,37 @@ ZTabArgs ztab_args(const vofp_plan* pl) {
   zt.za = pl->zaT;
   zt.lowcut = pl->lowcut;
   return zt;
+}
+
+ZCircArgs zcirc_args(const vofp_plan* pl) {
+  ZCircArgs zc;
+  zc.Ux = pl->Ux;
+  zc.bcx = pl->bc[0];
+  zc.bcy = pl->bc[1];
+  zc.ti = pl->zcirc_ti;
+  zc.L = pl->zcirc_rows;
+  zc.tab = pl->zcirc;
+  zc.lowcut = pl->lowcut;
+  return zc;
+}
+
+int build_zcirc(vofp_plan* pl, cudaStream_t st, bool sync) {
+  const ZArgs za = z_args(pl, false);
+  const ZCircArgs zc = zcirc_args(pl);
+  const int nb = (pl->Ux * pl->Uy + 127) / 128;
+  const double h = pl->dz_host[0];
+  if (pl->opts.prec == VOFP_MIXED)
+    k_zcirc_table<<<nb, 128, 0, st>>>(za, zc, pl->Uy, h, (ZCirc<float>*)pl->zcirc);
+  else if (pl->opts.prec == VOFP_FF)
+    k_zcirc_table<<<nb, 128, 0, st>>>(za, zc, pl->Uy, h, (ZCirc<ff>*)pl->zcirc);
+  else
+    k_zcirc_table<<<nb, 128, 0, st>>>(za, zc, pl->Uy, h, (ZCirc<double>*)pl->zcirc);
+  if (pl->zcirc_low)
+    k_zcirc_low_table<<<(pl->nlow + 127) / 128, 128, 0, st>>>(za, pl->lowmodes, pl->nlow, h,
+                                                             (ZCirc<double>*)pl->zcirc_low);
+  if (cudaGetLastError() != cudaSuccess) return VOFP_ERR_CUDA;
+  if (sync && cudaStreamSynchronize(st) != cudaSuccess) return VOFP_ERR_CUDA;
+  return VOFP_OK;
 }
 
 int build_z_factors(vofp_plan* pl, cudaStream_t st, bool sync) {
@@ -248,6 +280,11 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
     const dim3 tgrid((nx + zs.threads - 1) / zs.threads, ny);
     VOFP_LAUNCH(KID_ZSOLVE, st,
                 (k_ztab<double, ZF<double>><<<tgrid, zs.threads, zs.smem, st>>>(za, ztab_args(pl), zs.smem_d)));
+  } else if (pl->zcirc) {
+    const ZCircArgs zc = zcirc_args(pl);
+    const dim3 tgrid((nx + zc.ti - 1) / zc.ti, ny);
+    VOFP_LAUNCH(KID_ZSOLVE, st,
+                (k_zcirc<double><<<tgrid, kZCircThreads, zcirc_smem(nz, zc.ti, sizeof(double)), st>>>(za, zc)));
   } else {
     const int nvec = pl->bc[2] == VOFP_BC_P ? 3 : 2;
     const size_t zsm = (size_t)nvec * za.ti * nz * sizeof(double);

@@ -67,7 +67,7 @@ struct PlanLayout {
   size_t lam[2], tw[2], q[2], tw32[2], q32[2], twff[2], qff[2], blu64[2], blu32[2], bluff[2];
   size_t za, zb, zc, dz, hz, rdz, rhz, rzc, conv, info, low, za32, zaff, lowcut, kz, volf, dzff;
   size_t table_bytes;  // host-built part, uploaded as one copy
-  size_t P, S, T, S32, F, lowscr, lowtab, xtc;
+  size_t P, S, T, S32, F, lowscr, lowtab, zcirc, zcirc_low, xtc;
   size_t total;
 };
 struct PlanPrep {
@@ -94,6 +94,8 @@ GridDev grid_dev(const vofp_plan* pl);
 ZArgs z_args(const vofp_plan* pl, bool stats);
 struct ZTabArgs;
 ZTabArgs ztab_args(const vofp_plan* pl);
+struct ZCircArgs;
+ZCircArgs zcirc_args(const vofp_plan* pl);
 int grid_blocks(size_t total, int threads);
 void init_kernel_attributes_fp64();
 void init_kernel_attributes_mixed();
@@ -120,6 +122,8 @@ int mixed_solve(vofp_plan* pl, int mode, const XArgs* xa, const double* f, doubl
 int begin_info(vofp_plan* pl, cudaStream_t st, vofp_info* info);
 // Thomas factor tables for a bounded z axis (in the plan's arithmetic type), built on `st`; `sync` waits.
 int build_z_factors(vofp_plan* pl, cudaStream_t st, bool sync);
+// Periodic z with equal widths: the circulant systems' factors (zcirc.cuh), built on `st`; `sync` waits.
+int build_zcirc(vofp_plan* pl, cudaStream_t st, bool sync);
 // The same for the low-eigenvalue systems of a mixed plan.
 int build_low_factors(vofp_plan* pl, cudaStream_t st, bool sync);
 int finish_info(vofp_plan* pl, cudaStream_t st, vofp_info* info, int status);

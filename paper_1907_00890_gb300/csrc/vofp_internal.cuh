@@ -653,6 +653,11 @@ struct vofp_plan {
   void* ztab;    // bounded z: Thomas factors per distinct eigenvalue pair in the plan's arithmetic type
                  // (double2, float2 or cff; NULL: periodic z)
   const void* zaT;     // z sub-diagonal a_k in the same type
+  // periodic z with equal widths: the circulant systems' factors per distinct eigenvalue pair (arithmetic type),
+  // those of the low modes (FP64), columns per tile and rows per segment (see zcirc.cuh); NULL otherwise
+  void* zcirc;
+  void* zcirc_low;
+  int zcirc_ti, zcirc_rows;
   int* lowcut;         // refinement plans: spectral x index i of row j is a low mode iff i < lowcut[j]
   int Ux, Uy;    // distinct eigenvalue counts in x, y
   // mixed path
