@@ -1,0 +1,131 @@
+// Host side of the fixed-point transform passes (fxfft.cuh): which kernel, tile and scaling a launch takes.  Included
+// by one translation unit per spectrum type (the kernels compile side by side).
+#pragma once
+
+#include "fxfft.cuh"
+#include "solve_internal.h"
+
+namespace vofp {
+
+template <typename K>
+static void fx_allow_smem(K kern) {
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+}
+
+// The kernel of a pass for a tile: compiled for lines of 32 .. 512 samples at their usual tile width, else the run-time
+// one.
+static int fx_lgn(const FxTables& f) {
+  const int n = f.fd.n;
+  if ((n & (n - 1)) || n < 32 || n > 512) return 0;
+  const int lgn = 31 - __builtin_clz((unsigned)n);
+  if (f.lgB != fx_ct_lgB(lgn)) return 0;
+  for (int s = 0; s < f.fd.nst; ++s)  // (an autotuned stage order keeps the run-time kernel)
+    if (f.fd.radix[s] != fx_radix(lgn, s)) return 0;
+  return lgn;
+}
+typedef void (*FxXFwd)(const XArgs, const FxTables);
+typedef void (*FxYPass)(const YArgs, const FxTables);
+typedef void (*FxXInv)(const XInvArgs, const FxTables);
+template <typename T, int LGN>
+static FxXFwd fx_xfwd_mode(int mode) {
+  switch (mode) {
+    case RHS_F: return k_xfwd_fx<T, RHS_F, LGN>;
+    case RHS_DIV: return k_xfwd_fx<T, RHS_DIV, LGN>;
+    case RHS_DIV_STEFAN: return k_xfwd_fx<T, RHS_DIV_STEFAN, 0>;
+    case RHS_RESID:  // (a refinement plan's)
+      if constexpr (std::is_same<T, ff>::value) return k_xfwd_fx<T, RHS_RESID, LGN>;
+      else return nullptr;
+    default: return nullptr;
+  }
+}
+template <typename T>
+static FxXFwd fx_xfwd_kernel(int mode, int lgn) {
+  switch (mode == RHS_DIV_STEFAN ? 0 : lgn) {
+    case 5: return fx_xfwd_mode<T, 5>(mode);
+    case 6: return fx_xfwd_mode<T, 6>(mode);
+    case 7: return fx_xfwd_mode<T, 7>(mode);
+    case 8: return fx_xfwd_mode<T, 8>(mode);
+    case 9: return fx_xfwd_mode<T, 9>(mode);
+    default: return fx_xfwd_mode<T, 0>(mode);
+  }
+}
+template <typename T>
+static FxYPass fx_ypass_kernel(bool inv, int lgn) {
+  switch (lgn) {
+    case 5: return inv ? k_ypass_fx<T, true, 5> : k_ypass_fx<T, false, 5>;
+    case 6: return inv ? k_ypass_fx<T, true, 6> : k_ypass_fx<T, false, 6>;
+    case 7: return inv ? k_ypass_fx<T, true, 7> : k_ypass_fx<T, false, 7>;
+    case 8: return inv ? k_ypass_fx<T, true, 8> : k_ypass_fx<T, false, 8>;
+    case 9: return inv ? k_ypass_fx<T, true, 9> : k_ypass_fx<T, false, 9>;
+    default: return inv ? k_ypass_fx<T, true, 0> : k_ypass_fx<T, false, 0>;
+  }
+}
+template <typename T>
+static FxXInv fx_xinv_kernel(int lgn) {
+  switch (lgn) {
+    case 5: return k_xinv_fx<T, 5>;
+    case 6: return k_xinv_fx<T, 6>;
+    case 7: return k_xinv_fx<T, 7>;
+    case 8: return k_xinv_fx<T, 8>;
+    case 9: return k_xinv_fx<T, 9>;
+    default: return k_xinv_fx<T, 0>;
+  }
+}
+template <typename T>
+void init_fx_attributes() {
+  for (int lgn : {0, 5, 6, 7, 8, 9}) {
+    for (int mode : {RHS_F, RHS_DIV, RHS_DIV_STEFAN, RHS_RESID})
+      if (fx_xfwd_kernel<T>(mode, lgn)) fx_allow_smem(fx_xfwd_kernel<T>(mode, lgn));
+    fx_allow_smem(fx_ypass_kernel<T>(false, lgn));
+    fx_allow_smem(fx_ypass_kernel<T>(true, lgn));
+    fx_allow_smem(fx_xinv_kernel<T>(lgn));
+  }
+}
+
+// Tables and tile of axis ax for tiles8 tiles of eight lines; false: the axis' length has no fixed-point form.
+static bool fx_tables(const vofp_plan* pl, int ax, long tiles8, int least, FxTables* f) {
+  const AxisDev& a = pl->ax[ax];
+  if (!a.twfx || !fx_desc(a.fd, &f->fd)) return false;
+  f->tw = (const fxtw*)a.twfx;
+  f->quart = (const fxq*)a.quartfx;
+  f->lgB = fx_lgB(a.n, tiles8, least);
+  f->st = (1 << f->lgB) + (ax == 0 ? 1 : 0);
+  return true;
+}
+
+template <typename T>
+bool fx_xfwd(vofp_plan* pl, int mode, const XArgs& xa, cudaStream_t st) {
+  FxTables f;
+  const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
+  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, &f)) return false;
+  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
+  const size_t sm = fx_smem(f.fd, f.lgB, f.st);
+  const int kid = mode == RHS_F ? KID_XFWD : (mode == RHS_DIV ? KID_XFWD_DIV : (mode == RHS_RESID ? KID_RESID : KID_XFWD_DIVSTEF));
+  const FxXFwd kern = mode == RHS_STEFAN ? nullptr : fx_xfwd_kernel<T>(mode, fx_lgn(f));
+  if (!kern) return false;
+  VOFP_LAUNCH(kid, st, (kern<<<grid, th, sm, st>>>(xa, f)));
+  return true;
+}
+template <typename T>
+bool fx_ypass(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st) {
+  FxTables f;
+  const int nx = pl->n[0], nz = pl->n[2];
+  if (!fx_tables(pl, 1, (long)((nx + 15) / 16) * nz, 1, &f)) return false;
+  const dim3 grid((nx + (2 << f.lgB) - 1) / (2 << f.lgB), nz);
+  const int th = fx_threads(f.fd.n, f.lgB);
+  const size_t sm = fx_smem(f.fd, f.lgB, f.st);
+  VOFP_LAUNCH(inv ? KID_YINV : KID_YFWD, st, (fx_ypass_kernel<T>(inv, fx_lgn(f))<<<grid, th, sm, st>>>(ya, f)));
+  return true;
+}
+template <typename T>
+bool fx_xinv(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
+  FxTables f;
+  const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
+  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, &f)) return false;
+  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
+  const size_t sm = fx_smem(f.fd, f.lgB, f.st);
+  VOFP_LAUNCH(KID_XINV, st, (fx_xinv_kernel<T>(fx_lgn(f))<<<grid, th, sm, st>>>(xi, f)));
+  return true;
+}
+
+}  // namespace vofp

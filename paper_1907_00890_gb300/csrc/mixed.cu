@@ -305,6 +305,13 @@ struct Red<ff> {
   static const void* blu(const AxisDev& a) { return a.bluff; }
 };
 
+// The FP32-pair spectra's fixed-point y pass; false: not applicable.
+template <typename R>
+static bool ypass_fx(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st) {
+  if constexpr (std::is_same<R, ff>::value) return fx_ypass<ff>(pl, ya, inv, st);
+  else return false;
+}
+
 // y forward, z (bulk + FP64 low modes), y inverse on the spectrum; skipped when converged.
 template <typename R>
 static void solve_red(vofp_plan* pl, cudaStream_t st, int skip_k, double tol2, bool stats) {
@@ -326,7 +333,7 @@ static void solve_red(vofp_plan* pl, cudaStream_t st, int skip_k, double tol2, b
   ya.tol2 = tol2;
   const dim3 ygrid((nx + ya.tx - 1) / ya.tx, nz);
   const size_t ysm = 2 * (size_t)(ya.tx / 2) * y_ld(fft_span(ya.fd, ya.blu)) * sizeof(C);
-  if (ny > 1 && !ypass_tma<R>(pl, ya, false, st))
+  if (ny > 1 && !ypass_tma<R>(pl, ya, false, st) && !ypass_fx<R>(pl, ya, false, st))
     VOFP_LAUNCH(KID_YFWD, st, (ypass_kernel<R, C, false>()<<<ygrid, 256, ysm, st>>>(ya)));
   ZArgs za = z_args(pl, stats);
   za.S = pl->S32;
@@ -382,7 +389,7 @@ static void solve_red(vofp_plan* pl, cudaStream_t st, int skip_k, double tol2, b
                   k_zlow64<R><<<(pl->nlow + 63) / 64, 64, 0, st>>>(za, pl->lowmodes, pl->nlow, nullptr,
                                                                    pl->lowscratch));
   }
-  if (ny > 1 && !ypass_tma<R>(pl, ya, true, st))
+  if (ny > 1 && !ypass_tma<R>(pl, ya, true, st) && !ypass_fx<R>(pl, ya, true, st))
     VOFP_LAUNCH(KID_YINV, st, (ypass_kernel<R, C, true>()<<<ygrid, 256, ysm, st>>>(ya)));
 }
 
@@ -414,6 +421,9 @@ static void xinv_red(vofp_plan* pl, double* pout, int accumulate, int skip_k, do
   xi.mean_out = (pout && pl->singular && pl->opts.prec == VOFP_MIXED) ? pl->conv + VOFP_CONV_MEAN : nullptr;
   xi.d2_out = d2_out;
   if (std::is_same<R, float>::value && xtc_xinv(pl, xi, st)) return;  // tensor-core transform
+  if constexpr (std::is_same<R, ff>::value) {
+    if (fx_xinv<ff>(pl, xi, st)) return;  // fixed point
+  }
   if (xinv_tma<R>(pl, xi, st)) return;                                   // TMA-staged tiles
   const int xgrid = xpass_blocks(xi.ny, xi.nz, xi.pb);
   const size_t xsm = 2 * (size_t)xi.pb * fft_span(xi.fd, xi.blu) * sizeof(C);
@@ -431,6 +441,9 @@ static void xfwd_red(vofp_plan* pl, int mode, XArgs xa, cudaStream_t st) {
   xa.pb = pl->xpb;
   xa.S = pl->S32;
   if (std::is_same<R, float>::value && xtc_xfwd(pl, mode, xa, st)) return;  // tensor-core transform
+  if constexpr (std::is_same<R, ff>::value) {
+    if (fx_xfwd<ff>(pl, mode, xa, st)) return;  // fixed point
+  }
   const int xgrid = xpass_blocks(pl->n[1], pl->n[2], xa.pb);
   const size_t xsm = 2 * (size_t)xa.pb * fft_span(xa.fd, xa.blu) * sizeof(C);
   switch (mode) {

@@ -98,7 +98,7 @@ __device__ __forceinline__ double rhs_at(const XArgs& a, int i, int j, int k, do
   double f;
   if (MODE == RHS_F) {
     f = __ldg(a.f + c);
-    if (a.scale != 1.0) f *= a.scale;
+    if (__double_as_longlong(a.scale) != 0x3ff0000000000000ll) f *= a.scale;  // (integer test of 1.0)
   } else if (MODE == RHS_DIV) {
     f = divergence_at(a.g, a.u, a.v, a.w, i, j, k, a.src ? -__ldg(a.src + c) : 0.0) * a.scale;
   } else if (MODE == RHS_STEFAN) {

@@ -17,9 +17,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "solve_internal.h"
+#include "fxfft.cuh"
 #include "zcirc.cuh"
 #include "vofp_internal.cuh"
 
@@ -139,6 +141,36 @@ static std::vector<double2> bluestein_tables(const FftDesc& fd) {
   return t;
 }
 
+// cos and sin of pi p / q in Q62 (error below a unit): reduced to the first octant in integers, then the power series
+// in 64-bit fixed point.
+static void cis_q62(long long p, long long q, long long* c, long long* s) {
+  p %= 2 * q;
+  if (p < 0) p += 2 * q;
+  // angle pi p / q = pi/2 * quad + pi r / (4 q) with 0 <= r < 2q; beyond an eighth turn the roles swap
+  const long long p4 = 4 * p;
+  const int quad = (int)(p4 / (2 * q));
+  long long r = p4 - 2 * q * quad;  // in units of pi / (4 q)
+  const bool swap = r > q;
+  if (swap) r = 2 * q - r;
+  const unsigned long long piq62 = 0xC90FDAA22168C235ull;  // pi 2^62
+  const unsigned long long x = (unsigned long long)((unsigned __int128)piq62 * (unsigned long long)r / (4ull * q));
+  const unsigned long long x2 = (unsigned long long)((unsigned __int128)x * x >> 62);
+  unsigned long long one = 1ull << 62, tc = one, ts = x;
+  long long cs = (long long)one, sn = (long long)x;
+  for (int k = 1; k < 14; ++k) {
+    tc = (unsigned long long)((unsigned __int128)tc * x2 >> 62) / (unsigned)((2 * k - 1) * (2 * k));
+    ts = (unsigned long long)((unsigned __int128)ts * x2 >> 62) / (unsigned)((2 * k) * (2 * k + 1));
+    cs += (k & 1) ? -(long long)tc : (long long)tc;
+    sn += (k & 1) ? -(long long)ts : (long long)ts;
+  }
+  if (swap) std::swap(cs, sn);
+  switch (quad) {
+    case 0: *c = cs; *s = sn; break;
+    case 1: *c = -sn; *s = cs; break;
+    case 2: *c = -cs; *s = -sn; break;
+    default: *c = sn; *s = -cs; break;
+  }
+}
 static std::atomic<unsigned long long> g_launches{0};
 // While this thread captures a graph its launches are not executions: count them apart (they are added
 // once per replay instead) and do not trace them.
@@ -229,6 +261,8 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
   std::vector<double2> tw[2], quart[2];
   std::vector<float2> tw32[2], quart32[2];
   std::vector<cff> twff[2], quartff[2];
+  std::vector<fxtw> twfx[2];  // fixed-point tables (FP64 and FP32-pair plans, lengths without a Bluestein form)
+  std::vector<fxq> quartfx[2];
   std::vector<double2> blu[2];  // Bluestein tables (empty when the axis needs none)
   auto to_cff = [](double2 z) {
     cff c;
@@ -266,6 +300,23 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     p->ax[a].n = n;
     p->ax[a].bc = bc[a];
     if (p->ax[a].fd.bm) blu[a] = bluestein_tables(p->ax[a].fd);
+    FxDesc fx;
+    if (o.prec != VOFP_MIXED && fx_desc(p->ax[a].fd, &fx)) {
+      twfx[a].resize(n);
+      quartfx[a].resize(nq);
+      for (int q = 0; q < n; ++q) {
+        long long c, s;
+        cis_q62(2 * q, n, &c, &s);
+        twfx[a][q] = fx_twiddle(c, -s);
+      }
+      for (int q = 0; q < nq; ++q) {
+        long long c, s;
+        if (!quarter_bc(bc[a])) cis_q62(q, 2 * n, &c, &s);
+        else if (q < n) cis_q62(q, n, &c, &s);
+        else cis_q62(2 * (q - n) + 1, 4 * n, &c, &s);
+        quartfx[a][q] = {fx_weight(c), fx_weight(-s)};
+      }
+    }
   }
   std::vector<double> za(nz), zb(nz), zc(nz), hz(nz + 1), rdz(nz), rhz(nz + 1), rzc(nz), kz(4 * (size_t)nz);
   const double hper = 0.5 * (dz[nz - 1] + dz[0]);
@@ -344,6 +395,13 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     off = align256(off + sizeof(cff) * nn[a]);
     L.qff[a] = off;
     off = align256(off + sizeof(cff) * quartff[a].size());
+    L.twfx[a] = L.qfx[a] = 0;
+    if (!twfx[a].empty()) {
+      L.twfx[a] = off;
+      off = align256(off + sizeof(fxtw) * twfx[a].size());
+      L.qfx[a] = off;
+      off = align256(off + sizeof(fxq) * quartfx[a].size());
+    }
     L.blu64[a] = L.blu32[a] = L.bluff[a] = 0;
     if (!blu[a].empty()) {
       L.blu64[a] = off;
@@ -453,6 +511,10 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     memcpy(&host[L.q32[a]], quart32[a].data(), sizeof(float2) * quart32[a].size());
     memcpy(&host[L.twff[a]], twff[a].data(), sizeof(cff) * nn[a]);
     memcpy(&host[L.qff[a]], quartff[a].data(), sizeof(cff) * quartff[a].size());
+    if (!twfx[a].empty()) {
+      memcpy(&host[L.twfx[a]], twfx[a].data(), sizeof(fxtw) * twfx[a].size());
+      memcpy(&host[L.qfx[a]], quartfx[a].data(), sizeof(fxq) * quartfx[a].size());
+    }
     if (!blu[a].empty()) {
       const size_t m = blu[a].size();
       memcpy(&host[L.blu64[a]], blu[a].data(), sizeof(double2) * m);
@@ -574,6 +636,8 @@ int plan_bind(PlanPrep* pp, void* block, cudaStream_t st, unsigned char* stage) 
     p->ax[a].quart32 = (const float2*)(b + L.q32[a]);
     p->ax[a].twff = (const cff*)(b + L.twff[a]);
     p->ax[a].quartff = (const cff*)(b + L.qff[a]);
+    p->ax[a].twfx = L.twfx[a] ? (const void*)(b + L.twfx[a]) : nullptr;
+    p->ax[a].quartfx = L.qfx[a] ? (const void*)(b + L.qfx[a]) : nullptr;
     p->ax[a].blu64 = L.blu64[a] ? (const double2*)(b + L.blu64[a]) : nullptr;
     p->ax[a].blu32 = L.blu32[a] ? (const float2*)(b + L.blu32[a]) : nullptr;
     p->ax[a].bluff = L.bluff[a] ? (const cff*)(b + L.bluff[a]) : nullptr;

@@ -76,6 +76,8 @@ void init_kernel_attributes_fp64() {
   allow_smem(k_zsolve<double, double>);
   allow_smem(k_ztab<double, ZF<double>>);
   allow_smem(k_zcirc<double>);
+  init_fx_attributes<double>();
+  init_fx_attributes<ff>();
   allow_smem(k_ztab_staged<double, ZF<double>>);
   allow_smem(k_ztab_seg<double, ZF<double>, false>);
   allow_smem(k_ztab_seg<double, ZF<double>, true>);
@@ -233,7 +235,7 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
   const long npairs = ((long)ny * nz + 1) / 2;
   const int xgrid = (int)((npairs + xa.pb - 1) / xa.pb);
   const size_t xsm = 2 * (size_t)xa.pb * fft_span(xa.fd, xa.blu) * sizeof(double2);
-  switch (mode) {
+  if (!fx_xfwd<double>(pl, mode, xa, st)) switch (mode) {
     case RHS_F: VOFP_LAUNCH(KID_XFWD, st, k_xfwd_f64<RHS_F><<<xgrid, 256, xsm, st>>>(xa)); break;
     case RHS_DIV: VOFP_LAUNCH(KID_XFWD_DIV, st, k_xfwd_f64<RHS_DIV><<<xgrid, 256, xsm, st>>>(xa)); break;
     case RHS_STEFAN:
@@ -258,7 +260,7 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
   ya.S = pl->S;
   const dim3 ygrid((nx + ya.tx - 1) / ya.tx, nz);
   const size_t ysm = 2 * (size_t)(ya.tx / 2) * y_ld(fft_span(ya.fd, ya.blu)) * sizeof(double2);
-  if (ny > 1 && !ypass_tma_f64(pl, ya, false, st))
+  if (ny > 1 && !fx_ypass<double>(pl, ya, false, st) && !ypass_tma_f64(pl, ya, false, st))
     VOFP_LAUNCH(KID_YFWD, st, k_ypass_f64<false><<<ygrid, 256, ysm, st>>>(ya));
   ZArgs za = z_args(pl, stats);
   if (pl->ztab && (pl->zti == -1 || pl->zti == -2)) {  // (only by the autotuner's choice on FP64 plans)
@@ -291,7 +293,7 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
     const dim3 zgrid((nx + za.ti - 1) / za.ti, ny);
     VOFP_LAUNCH(KID_ZSOLVE, st, (k_zsolve<double, double><<<zgrid, 128, zsm, st>>>(za)));
   }
-  if (ny > 1 && !ypass_tma_f64(pl, ya, true, st))
+  if (ny > 1 && !fx_ypass<double>(pl, ya, true, st) && !ypass_tma_f64(pl, ya, true, st))
     VOFP_LAUNCH(KID_YINV, st, k_ypass_f64<true><<<ygrid, 256, ysm, st>>>(ya));
   XInvArgs xi = {};
   xi.skip_k = -1;
@@ -307,7 +309,7 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
   xi.S = pl->S;
   xi.p = pout;
   xi.accumulate = 0;
-  VOFP_LAUNCH(KID_XINV, st, k_xinv_f64<0><<<xgrid, 256, xsm, st>>>(xi));
+  if (!fx_xinv<double>(pl, xi, st)) VOFP_LAUNCH(KID_XINV, st, k_xinv_f64<0><<<xgrid, 256, xsm, st>>>(xi));
   return cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
 }
 

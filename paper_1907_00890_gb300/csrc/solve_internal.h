@@ -64,7 +64,7 @@ unsigned long long capture_end();
 
 // ---- plan construction in two phases (see plan.cu) ----
 struct PlanLayout {
-  size_t lam[2], tw[2], q[2], tw32[2], q32[2], twff[2], qff[2], blu64[2], blu32[2], bluff[2];
+  size_t lam[2], tw[2], q[2], tw32[2], q32[2], twff[2], qff[2], blu64[2], blu32[2], bluff[2], twfx[2], qfx[2];
   size_t za, zb, zc, dz, hz, rdz, rhz, rzc, conv, info, low, za32, zaff, lowcut, kz, volf, dzff;
   size_t table_bytes;  // host-built part, uploaded as one copy
   size_t P, S, T, S32, F, lowscr, lowtab, zcirc, zcirc_low, xtc;
@@ -106,6 +106,16 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
 // The FP64 plans' y pass on TMA-staged tiles when applicable (power-of-two ny; mixed.cu); false: not run.
 struct YArgs;
 bool ypass_tma_f64(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st);
+// The fixed-point transform passes of FP64 (T = double) and FP32-pair (T = ff) spectra (fxpass.cuh, instantiated in
+// fx64.cu and fxff.cu); false: the axis' length has none (a Bluestein length, a plan without the tables), not run.
+template <typename T>
+void init_fx_attributes();
+template <typename T>
+bool fx_xfwd(vofp_plan* pl, int mode, const XArgs& xa, cudaStream_t st);
+template <typename T>
+bool fx_ypass(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st);
+template <typename T>
+bool fx_xinv(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st);
 // The plan's FP64 x transform (forward, or inverse) of nlines lines `in` -> `out` (see solve.cu).
 int fp64_x_lines(vofp_plan* pl, bool inverse, const double* in, double* out, int nlines, cudaStream_t st);
 // Tensor-core x passes of FP32 refinement plans (xtc.cu): table sizes at plan preparation, the tables' build

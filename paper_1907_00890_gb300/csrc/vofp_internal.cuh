@@ -149,6 +149,9 @@ struct AxisDev {
   const double2* blu64;  // Bluestein tables (see fft_smem), NULL when n needs none
   const float2* blu32;
   const cff* bluff;
+  // fixed-point twiddles and quarter-wave twiddles (fxfft.cuh; FP64 and FP32-pair plans), NULL: the length has none
+  const void* twfx;
+  const void* quartfx;
   const double* lam; // eigenvalue of packed spectral index q, q < n
 };
 
