@@ -170,21 +170,17 @@ __global__ void k_shift_batch(const EpiArgs* __restrict__ e, const int* __restri
   for (size_t t = (size_t)l * blockDim.x + threadIdx.x; t < cells; t += (size_t)nb * blockDim.x) a.p[t] -= m;
 }
 
-// Velocity correction of every instance: up to 512 blocks per instance striding over its faces (the
-// instance lookup, a dependent binary search, is paid once per block: a block per 256 faces made it the
-// kernel's cost).
+// Velocity correction of every instance: up to 512 blocks per instance striding over its corner tiles (the instance
+// lookup, a dependent binary search, is paid once per block).
 __global__ void k_grad_batch(const EpiArgs* __restrict__ e, const int* __restrict__ off, int n) {
   const int inst = find_instance(off, n, blockIdx.x);
   const EpiArgs& a = e[inst];
   const int nb = __ldg(off + inst + 1) - __ldg(off + inst);
-  const int l = blockIdx.x - __ldg(off + inst);
   const GridDev g = a.g;
-  const size_t total = total_faces(g);
-  for (size_t t = (size_t)l * blockDim.x + threadIdx.x; t < total; t += (size_t)nb * blockDim.x) {
-    int i, j, k;
-    size_t o;
-    const int axis = decode_face(g, t, i, j, k, o);
-    if (VOFP_IN(o, nfaces(g, axis), CHK_FACE_STORE)) grad_face(g, a.p, a.u, a.v, a.w, a.s, a.sx, a.sy, axis, i, j, k, o);
+  const int tx = corner_tiles_x(g), txy = tx * corner_tiles_y(g), tiles = txy * nface(g.nz, g.bcz);
+  for (int t = blockIdx.x - __ldg(off + inst); t < tiles; t += nb) {
+    const int k = t / txy, r = t - k * txy, ty = r / tx;
+    grad_tile(g, a.p, a.u, a.v, a.w, a.s, a.sx, a.sy, r - ty * tx, ty, k);
   }
 }
 

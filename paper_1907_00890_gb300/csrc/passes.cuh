@@ -34,7 +34,7 @@ struct XArgs {
   const double* C;
   const double* mdot;
   const double* p;    // RHS_RESID: current potential
-  double scale;       // multiplies the right-hand side (RHS_F, RHS_DIV)
+  double scale;       // multiplies the right-hand side (RHS_DIV, RHS_DIV_STEFAN)
   double coef;        // RHS_STEFAN: 1/rho2 - 1/rho1
   int grad_mode;
   double* fsave;      // if non-null, the FP64 right-hand side is stored here (mixed path)
@@ -98,7 +98,6 @@ __device__ __forceinline__ double rhs_at(const XArgs& a, int i, int j, int k, do
   double f;
   if (MODE == RHS_F) {
     f = __ldg(a.f + c);
-    if (__double_as_longlong(a.scale) != 0x3ff0000000000000ll) f *= a.scale;  // (integer test of 1.0)
   } else if (MODE == RHS_DIV) {
     f = divergence_at(a.g, a.u, a.v, a.w, i, j, k, a.src ? -__ldg(a.src + c) : 0.0) * a.scale;
   } else if (MODE == RHS_STEFAN) {

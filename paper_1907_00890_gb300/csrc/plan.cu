@@ -708,12 +708,14 @@ int ensure_geometry(vofp_plan* p) {
   if (p->G) return VOFP_OK;
   const size_t cells = (size_t)p->n[0] * p->n[1] * p->n[2];
   void* m = nullptr;
-  if (device_alloc(&m, 4 * sizeof(double) * cells) != cudaSuccess) {
+  // s and n, then a mask word per 32 cells of a row (see k_geometry)
+  const size_t bytes = 4 * sizeof(double) * cells + sizeof(unsigned) * (size_t)((p->n[0] + 31) / 32) * p->n[1] * p->n[2];
+  if (device_alloc(&m, bytes) != cudaSuccess) {
     cudaGetLastError();
     return VOFP_ERR_OOM;
   }
   p->G = (double*)m;
-  p->bytes += 4 * sizeof(double) * cells;
+  p->bytes += bytes;
   return VOFP_OK;
 }
 

@@ -351,16 +351,17 @@ static int launch_geometry(vofp_plan* pl, const double* C, const double* mdot, d
   double* G = pl->G;
   const int mode = pl->opts.grad_mode;
   double* sp = s_out ? s_out : G;
+  unsigned* mask = with_n ? (unsigned*)(G + 4 * cells) : nullptr;
   double* n0 = with_n ? G + cells : nullptr;
   double* n1 = with_n ? G + 2 * cells : nullptr;
   double* n2 = with_n ? G + 3 * cells : nullptr;
-  const int th = g.nx >= 128 ? 128 : 64;
+  const dim3 grid = geometry_grid(g);
   if (mode == 0 && pl->opts.prec != VOFP_FP64)  // reduced-precision plans: FP32-pair geometry
-    VOFP_LAUNCH(KID_STEFAN, st, k_geometry_ff<<<cell_grid(g, th), th, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2));
+    VOFP_LAUNCH(KID_STEFAN, st, (k_geometry<0, true><<<grid, 128, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2, mask)));
   else if (mode == 1)
-    VOFP_LAUNCH(KID_STEFAN, st, k_geometry<1><<<cell_grid(g, th), th, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2));
+    VOFP_LAUNCH(KID_STEFAN, st, (k_geometry<1, false><<<grid, 128, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2, mask)));
   else
-    VOFP_LAUNCH(KID_STEFAN, st, k_geometry<0><<<cell_grid(g, th), th, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2));
+    VOFP_LAUNCH(KID_STEFAN, st, (k_geometry<0, false><<<grid, 128, 0, st>>>(g, C, mdot, coef, sp, n0, n1, n2, mask)));
   return cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
 }
 
@@ -379,8 +380,8 @@ static int project_common(vofp_plan* pl, int mode, XArgs& xa, double* u, double*
   }
   const GridDev g = grid_dev(pl);
   VOFP_LAUNCH(KID_GRAD, st,
-              k_grad_update<<<face_grid(g, 256), 256, 0, st>>>(g, pout, u, v, w, dt_over_rho0,
-                                                                      dt_over_rho0 * g.rdx, dt_over_rho0 * g.rdy));
+              k_grad_update<<<corner_grid(g), corner_threads(g), 0, st>>>(g, pout, u, v, w, dt_over_rho0, dt_over_rho0 * g.rdx,
+                                                                      dt_over_rho0 * g.rdy));
   const int ls = cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
   if (pl->opts.prec != VOFP_FP64) {
     if (ls) return ls;
@@ -423,6 +424,7 @@ static int extend_common(vofp_plan* pl, const double* u, const double* v, const 
   ea.n[0] = pl->G + cells;
   ea.n[1] = pl->G + 2 * cells;
   ea.n[2] = pl->G + 3 * cells;
+  ea.mask = (const unsigned*)(pl->G + 4 * cells);
   ea.quarter_inv_rho1 = 0.25 / rho_ext;
   ea.ue = ue;
   ea.ve = ve;
@@ -430,7 +432,7 @@ static int extend_common(vofp_plan* pl, const double* u, const double* v, const 
   ea.ug = ug;
   ea.vg = vg;
   ea.wg = wg;
-  VOFP_LAUNCH(KID_EXTEND_EPI, st, k_extend_epi<<<face_grid(ea.g, 256), 256, 0, st>>>(ea));
+  VOFP_LAUNCH(KID_EXTEND_EPI, st, k_extend_epi<<<corner_grid(ea.g), corner_threads(ea.g), 0, st>>>(ea));
   const int ls = cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
   if (pl->opts.prec != VOFP_FP64) {
     if (ls) return ls;
@@ -501,7 +503,7 @@ extern "C" int vofp_project_vd(vofp_plan* pl, double* u, double* v, double* w, c
   va.u = u;
   va.v = v;
   va.w = w;
-  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<face_grid(va.g, 256), 256, 0, st>>>(va));
+  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<corner_grid(va.g), corner_threads(va.g), 0, st>>>(va));
   if (cudaGetLastError() != cudaSuccess) return VOFP_ERR_CUDA;
   return vofp_project(pl, u, v, w, src, dt / rho0, p, stream, info);
 }

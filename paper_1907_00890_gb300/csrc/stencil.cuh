@@ -78,6 +78,24 @@ __device__ __forceinline__ double cval(const GridDev& g, const double* __restric
   return ldg_in(C, ((size_t)k * g.ny + j) * g.nx + i, ncells(g), CHK_CELL_LOAD);
 }
 
+// Youngs' corner average at the middle of the 3 x 3 cells (x fastest) m, c, p of planes k - 1, k, k + 1: differences first
+// (C near 0 or 1 loses nothing in them), then the (1, 2, 1) / 4 filter of both transverse directions by the sums of the
+// corner (weight 1), edge (2) and middle (4) differences; on a uniform axis the two one-sided differences add up to one
+// over two cells.
+__device__ __forceinline__ double3 youngs_gradient(const GridDev& g, const double* m, const double* c, const double* p,
+                                                   int k) {
+  const double x = fma(4.0, c[5] - c[3], fma(2.0, ((c[2] - c[0]) + (c[8] - c[6])) + ((m[5] - m[3]) + (p[5] - p[3])),
+                                             ((m[2] - m[0]) + (m[8] - m[6])) + ((p[2] - p[0]) + (p[8] - p[6]))));
+  const double y = fma(4.0, c[7] - c[1], fma(2.0, ((c[6] - c[0]) + (c[8] - c[2])) + ((m[7] - m[1]) + (p[7] - p[1])),
+                                             ((m[6] - m[0]) + (m[8] - m[2])) + ((p[6] - p[0]) + (p[8] - p[2]))));
+  auto z = [](const double* lo, const double* hi) {
+    return fma(4.0, hi[4] - lo[4], fma(2.0, ((hi[1] - lo[1]) + (hi[7] - lo[7])) + ((hi[3] - lo[3]) + (hi[5] - lo[5])),
+                                       ((hi[0] - lo[0]) + (hi[2] - lo[2])) + ((hi[6] - lo[6]) + (hi[8] - lo[8]))));
+  };
+  return make_double3(0.03125 * g.rdx * x, 0.03125 * g.rdy * y,
+                      0.03125 * fma(z(m, c), __ldg(g.rhz + k), z(c, p) * __ldg(g.rhz + k + 1)));
+}
+
 // Cell-centred gradient of C: mode 0 central, mode 1 Youngs.
 __device__ __forceinline__ double3 grad_c_at(const GridDev& g, const double* __restrict__ C, int i, int j, int k,
                                              int mode) {
@@ -88,50 +106,41 @@ __device__ __forceinline__ double3 grad_c_at(const GridDev& g, const double* __r
     r.z = (cval(g, C, i, j, k + 1) - cval(g, C, i, j, k - 1)) * __ldg(g.rzc + k);
     return r;
   }
-  const double wt[3] = {0.25, 0.5, 0.25};
-  double gx = 0, gy = 0, gz = 0;
-  for (int s = 0; s < 2; ++s) {
-    double ax = 0, ay = 0, az = 0;
-    for (int a = -1; a <= 1; ++a) {
-      for (int b = -1; b <= 1; ++b) {
-        const double wab = wt[a + 1] * wt[b + 1];
-        ax += wab * (cval(g, C, i + s, j + a, k + b) - cval(g, C, i + s - 1, j + a, k + b));
-        ay += wab * (cval(g, C, i + a, j + s, k + b) - cval(g, C, i + a, j + s - 1, k + b));
-        az += wab * (cval(g, C, i + a, j + b, k + s) - cval(g, C, i + a, j + b, k + s - 1));
-      }
-    }
-    gx += ax * g.rdx;
-    gy += ay * g.rdy;
-    gz += az * __ldg(g.rhz + k + s);
-  }
-  r.x = 0.5 * gx;
-  r.y = 0.5 * gy;
-  r.z = 0.5 * gz;
-  return r;
+  double q[3][9];
+  for (int b = -1; b <= 1; ++b)
+    for (int a = 0; a < 9; ++a) q[b + 1][a] = cval(g, C, i + a % 3 - 1, j + a / 3 - 1, k + b);
+  return youngs_gradient(g, q[0], q[1], q[2], k);
 }
 
-// |grad C| and the unit normal n = -grad C / |grad C| (zero where clipped) at one cell.
-__device__ __forceinline__ double geometry_at(const GridDev& g, const double* __restrict__ C, int i, int j, int k,
-                                              int mode, double3& n) {
-  const double3 gc = grad_c_at(g, C, i, j, k, mode);
+constexpr long long kClipHigh = 0x3feffffffaa19c47ll;  // the bits of the largest C with 1 - C >= 1e-8
+
+// 1 / sqrt(x) for x > 0: an FP32 seed of x's mantissa (exponent halved in integers, relative error below 2^-21) and one
+// third-order step, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2: error 5 e^3 / 16, five FP64 operations.
+__device__ __forceinline__ double rsqrt_step(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) - 1023;
+  if (e < -900 || e > 900) return rsqrt(x);  // (near the ends of the range, infinities and NaN)
+  const int odd = e & 1;
+  const unsigned m = __funnelshift_l((unsigned)__double2loint(x), (unsigned)hi, 3) & 0x7fffffu;
+  double y = f64_of_bits(rsqrtf(__uint_as_float(m | ((unsigned)(127 + odd) << 23))));
+  y = __hiloint2double(__double2hiint(y) - (((e - odd) / 2) << 20), __double2loint(y));
+  const double r = fma(-(x * y), y, 1.0);
+  return fma(y * r, fma(0.375, r, 0.5), y);
+}
+
+// |grad C| and the unit normal n = -grad C / |grad C| (zero where clipped) from a cell's gradient and its C.
+__device__ __forceinline__ double normal_of(double3 gc, double c, double3& n) {
   const double m2 = fma(gc.x, gc.x, fma(gc.y, gc.y, gc.z * gc.z));
   n = make_double3(0.0, 0.0, 0.0);
-  if (m2 == 0.0) return 0.0;
-  const double r = rsqrt(m2);
-  const double c = ldg_in(C, ((size_t)k * g.ny + j) * g.nx + i, ncells(g), CHK_CELL_LOAD);
-  if (fmin(c, 1.0 - c) >= 1e-8) {
+  if (__double_as_longlong(m2) == 0) return 0.0;
+  const double r = rsqrt_step(m2);
+  // min(C, 1 - C) >= 1e-8 by the bits of C: 1 - C is exact there, and kClipHigh the last such C
+  const long long b = __double_as_longlong(c);
+  if (b >= __double_as_longlong(1e-8) && b <= kClipHigh) {
     n.x = -gc.x * r;
     n.y = -gc.y * r;
     n.z = -gc.z * r;
   }
   return m2 * r;
-}
-
-__device__ __forceinline__ double3 normal_at(const GridDev& g, const double* __restrict__ C, int i, int j, int k,
-                                             int mode) {
-  double3 n;
-  geometry_at(g, C, i, j, k, mode, n);
-  return n;
 }
 
 }  // namespace vofp
