@@ -34,14 +34,6 @@ inline dim3 corner_grid(const GridDev& g) {
   return dim3((unsigned)corner_tiles_x(g), (unsigned)corner_tiles_y(g), (unsigned)nface(g.nz, g.bcz));
 }
 
-// Keeps what follows in one copy: the compiler would split FP64 instructions over the cases of a select, and one that is
-// predicated off still takes its turn on the FP64 pipe (the correction kernel issued 9.2 FP64 instructions a cell for
-// the six it needs).
-__device__ __forceinline__ double one_path(double x) {
-  asm volatile("" : "+d"(x));
-  return x;
-}
-
 // Double a normal value by its exponent.
 __device__ __forceinline__ double twice(double x) {
   return __hiloint2double(__double2hiint(x) + 0x100000, __double2loint(x));
@@ -129,15 +121,9 @@ static __global__ void __launch_bounds__(kCornerThreads) k_grad_update(GridDev g
 // with a gradient, 7% with a normal) 44.7 us, 71.7 before; FP32-pair plans 31.4 us, 43.4 before; Youngs' average on 96 x
 // 80 x 72 82.5 us, 154 before.
 __host__ __device__ __forceinline__ int mask_words(int nx) { return (nx + 31) >> 5; }
-__device__ __forceinline__ bool same_bits(double a, double b) {
-  return __double_as_longlong(a) == __double_as_longlong(b);
-}
-__device__ __forceinline__ bool finite_bits(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool any_bits(double a, double b, double c) {
   return ((__double_as_longlong(a) | __double_as_longlong(b) | __double_as_longlong(c)) << 1) != 0;
 }
-
-__device__ __forceinline__ bool same_value(double a, double b) { return same_bits(a, b) && finite_bits(a); }
 
 // Store n where it is not zero and the warp's mask word (lanes are 32 consecutive cells of a row, all active).  A cell
 // whose mdot is not finite is marked too: the face means then read it, as they would without the mask.

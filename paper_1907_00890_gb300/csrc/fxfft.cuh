@@ -193,9 +193,15 @@ static __device__ __noinline__ double fx_to_rare(long long v, int K) {
 __device__ __forceinline__ double fx_to(long long v, int K, int flip, double*) {
   const int vh = (int)(v >> 32);
   const unsigned long long a = (unsigned long long)(vh < 0 ? -v : v);
-  const unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
+  unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
+  int e = 1085 + K;  // one below the biased exponent: the implicit bit adds it
+  if (h == 0) {
+    h = l;
+    l = 0;
+    e -= 32;
+  }
   const int lz = __clz((int)h);
-  const int e = 1085 - lz + K;  // one below the biased exponent: the implicit bit adds it
+  e -= lz;
   if (h == 0 || (unsigned)e > 2044u) return ((v == 0 && K != kFxNan) || K == kFxZero) ? 0.0 : fx_to_rare(flip ? -v : v, K);
   const unsigned nh = __funnelshift_l(l, h, lz), nl = l << lz;
   const unsigned rh = (nh >> 11) + (((unsigned)e << 20) | ((unsigned)(vh ^ flip) & 0x80000000u));
@@ -1012,8 +1018,10 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_ypass_fx(cons
   }
 }
 
-// Inverse x transform into the FP64 cell array p (written, or added to; NULL: only its size in d2_out).
-template <typename T, int LGN>
+// Inverse x transform into the FP64 cell array p.  PLAIN: written, and nothing else; otherwise written or added to (NULL:
+// only its size in d2_out) with the sums asked for (as FP64 instructions that are predicated off, they cost the plain
+// pass three turns of the FP64 pipe a value: 24.8 -> 22.6 us at 128^3).
+template <typename T, int LGN, bool PLAIN>
 __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xinv_fx(const __grid_constant__ XInvArgs a,
                                                                         const __grid_constant__ FxTables f) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1077,6 +1085,10 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xinv_fx(const
     for (int h = 0; h < 2; ++h) {
       if (l + h >= nlines || !VOFP_IN(w + h * n, (size_t)nlines * n, CHK_XINV)) continue;
       const double v = fx_to(ov[h], Kb, 0, (double*)nullptr);
+      if (PLAIN) {
+        a.p[w + h * n] = v;
+        continue;
+      }
       if (a.p && !a.accumulate) a.p[w + h * n] = v;
       else if (a.p) a.p[w + h * n] += v;
       if (a.mean_out) acc = fma(v, __ldg(a.dz + (l + h) / a.ny), acc);
@@ -1098,6 +1110,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xinv_fx(const
       store(pb, i, fx_neg_if(y.x, fl), fx_neg_if(y.y, !fl));
     }
   }
+  if (PLAIN) return;
   if (a.mean_out) {
     const double s = block_sum(acc, red);
     if (threadIdx.x == 0 && s != 0) atomicAdd(a.mean_out, s);

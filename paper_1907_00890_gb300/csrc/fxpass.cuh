@@ -60,16 +60,23 @@ static FxYPass fx_ypass_kernel(bool inv, int lgn) {
     default: return inv ? k_ypass_fx<T, true, 0> : k_ypass_fx<T, false, 0>;
   }
 }
-template <typename T>
+template <typename T, bool PLAIN>
 static FxXInv fx_xinv_kernel(int lgn) {
   switch (lgn) {
-    case 5: return k_xinv_fx<T, 5>;
-    case 6: return k_xinv_fx<T, 6>;
-    case 7: return k_xinv_fx<T, 7>;
-    case 8: return k_xinv_fx<T, 8>;
-    case 9: return k_xinv_fx<T, 9>;
-    default: return k_xinv_fx<T, 0>;
+    case 5: return k_xinv_fx<T, 5, PLAIN>;
+    case 6: return k_xinv_fx<T, 6, PLAIN>;
+    case 7: return k_xinv_fx<T, 7, PLAIN>;
+    case 8: return k_xinv_fx<T, 8, PLAIN>;
+    case 9: return k_xinv_fx<T, 9, PLAIN>;
+    default: return k_xinv_fx<T, 0, PLAIN>;
   }
+}
+// (FP64 plans only ever write the potential)
+template <typename T>
+static FxXInv fx_xinv_kernel(int lgn, bool plain) {
+  if constexpr (!std::is_same<T, double>::value)
+    if (!plain) return fx_xinv_kernel<T, false>(lgn);
+  return plain ? fx_xinv_kernel<T, true>(lgn) : nullptr;
 }
 template <typename T>
 void init_fx_attributes() {
@@ -78,7 +85,8 @@ void init_fx_attributes() {
       if (fx_xfwd_kernel<T>(mode, lgn)) fx_allow_smem(fx_xfwd_kernel<T>(mode, lgn));
     fx_allow_smem(fx_ypass_kernel<T>(false, lgn));
     fx_allow_smem(fx_ypass_kernel<T>(true, lgn));
-    fx_allow_smem(fx_xinv_kernel<T>(lgn));
+    for (bool plain : {true, false})
+      if (fx_xinv_kernel<T>(lgn, plain)) fx_allow_smem(fx_xinv_kernel<T>(lgn, plain));
   }
 }
 
@@ -124,7 +132,9 @@ bool fx_xinv(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
   if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, &f)) return false;
   const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
-  VOFP_LAUNCH(KID_XINV, st, (fx_xinv_kernel<T>(fx_lgn(f))<<<grid, th, sm, st>>>(xi, f)));
+  const FxXInv kern = fx_xinv_kernel<T>(fx_lgn(f), xi.p && !xi.accumulate && !xi.mean_out && !xi.d2_out);
+  if (!kern) return false;
+  VOFP_LAUNCH(KID_XINV, st, (kern<<<grid, th, sm, st>>>(xi, f)));
   return true;
 }
 

@@ -67,7 +67,7 @@ __device__ __forceinline__ double resid_at(const GridDev& g, const double* __res
     else lo = g.bcx == VOFP_BC_P ? __ldg(p + c + g.nx - 1) : neg_if(pc, g.bcx == VOFP_BC_DD || g.bcx == VOFP_BC_DN);
     if (i < g.nx - 1) hi = __ldg(p + c + 1);
     else hi = g.bcx == VOFP_BC_P ? __ldg(p + c - (g.nx - 1)) : neg_if(pc, g.bcx == VOFP_BC_DD || g.bcx == VOFP_BC_ND);
-    xs = hi + lo;
+    xs = one_path(hi) + one_path(lo);
   }
   {
     double lo, hi;
@@ -77,7 +77,7 @@ __device__ __forceinline__ double resid_at(const GridDev& g, const double* __res
     if (j < g.ny - 1) hi = __ldg(p + c + g.nx);
     else hi = g.bcy == VOFP_BC_P ? __ldg(p + c - (size_t)(g.ny - 1) * g.nx)
                                  : neg_if(pc, g.bcy == VOFP_BC_DD || g.bcy == VOFP_BC_ND);
-    ys = hi + lo;
+    ys = one_path(hi) + one_path(lo);
   }
   {
     const bool lowN = g.bcz == VOFP_BC_NN || g.bcz == VOFP_BC_ND;
@@ -87,6 +87,8 @@ __device__ __forceinline__ double resid_at(const GridDev& g, const double* __res
     if (k < g.nz - 1) zhi = __ldg(p + c + plane);
     else zhi = g.bcz == VOFP_BC_P ? __ldg(p + c - (size_t)(g.nz - 1) * plane) : neg_if(pc, !highN);
   }
+  zlo = one_path(zlo);
+  zhi = one_path(zhi);
   return fma(-g.rdx2, xs,
              fma(-g.rdy2, ys, fma(-__ldg(g.czc + k), pc, fma(-__ldg(g.czp + k), zhi, fma(-__ldg(g.czm + k), zlo, base)))));
 }
@@ -99,7 +101,8 @@ __device__ __forceinline__ double rhs_at(const XArgs& a, int i, int j, int k, do
   if (MODE == RHS_F) {
     f = __ldg(a.f + c);
   } else if (MODE == RHS_DIV) {
-    f = divergence_at(a.g, a.u, a.v, a.w, i, j, k, a.src ? -__ldg(a.src + c) : 0.0) * a.scale;
+    const double s = one_path(a.src ? __ldg(a.src + c) : 0.0);  // (negated as an operand, not by an instruction)
+    f = divergence_at(a.g, a.u, a.v, a.w, i, j, k, -s) * a.scale;
   } else if (MODE == RHS_STEFAN) {
     const double3 gc = grad_c_at(a.g, a.C, i, j, k, a.grad_mode);
     f = __ldg(a.mdot + c) * a.coef * sqrt(gc.x * gc.x + gc.y * gc.y + gc.z * gc.z);
@@ -108,8 +111,7 @@ __device__ __forceinline__ double rhs_at(const XArgs& a, int i, int j, int k, do
     const double s = __ldg(a.mdot + c) * a.coef * sqrt(gc.x * gc.x + gc.y * gc.y + gc.z * gc.z);
     f = divergence_at(a.g, a.u, a.v, a.w, i, j, k, -s) * a.scale;
   } else {
-    // (fbar = 0 unless the operator is singular: no subtraction then)
-    f = resid_at(a.g, a.p, i, j, k, a.defect_sum ? __ldg(a.f + c) - fbar : __ldg(a.f + c));
+    f = resid_at(a.g, a.p, i, j, k, one_path(__ldg(a.f + c)) - fbar);
   }
   return f;
 }

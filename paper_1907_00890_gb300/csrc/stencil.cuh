@@ -35,6 +35,20 @@ struct GridDev {
   const ff* dzff;     // dz per plane, FP32 pair
 };
 
+__device__ __forceinline__ bool same_bits(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
+__device__ __forceinline__ bool finite_bits(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool same_value(double a, double b) { return same_bits(a, b) && finite_bits(a); }
+
+// Keeps what follows in one copy: the compiler would split FP64 instructions over the cases of a select, and one that is
+// predicated off still takes its turn on the FP64 pipe (the correction kernel issued 9.2 FP64 instructions a cell for
+// the six it needs).
+__device__ __forceinline__ double one_path(double x) {
+  asm volatile("" : "+d"(x));
+  return x;
+}
+
 __host__ __device__ __forceinline__ int nface(int n, int bc) { return n + (bc != VOFP_BC_P); }
 __host__ __device__ __forceinline__ size_t ncells(const GridDev& g) { return (size_t)g.nx * g.ny * g.nz; }
 // the u, v, w face arrays: nface cells along their own axis
