@@ -20,59 +20,6 @@
 
 namespace vofp {
 
-// Upwind value C_upwind across face f (the low face of cell f) of a line of n cells at `base` with stride
-// `st`, for the face velocity `vel`: the cell the flow comes from (sign bit of vel, an integer test; a zero
-// velocity of either sign gives a zero flux whichever cell is taken), beyond a bounded end the boundary cell.
-__device__ __forceinline__ double upwind_value(const double* __restrict__ q, size_t base, size_t st, int n, int bc,
-                                               int f, double vel) {
-  int lo = f - 1, hi = f;  // the cells across the face
-  if (bc == VOFP_BC_P) {
-    if (lo < 0) lo += n;
-    if (hi >= n) hi -= n;
-  } else {
-    if (lo < 0) lo = 0;
-    if (hi >= n) hi = n - 1;
-  }
-  return __ldg(q + base + (size_t)(__double2hiint(vel) >= 0 ? lo : hi) * st);
-}
-
-// One implicit directional step along `axis` for cell (i, j, k): returns the new value of q there and sets
-// `du` to the face-velocity difference over the cell width.  With dt factored out of the fluxes,
-//   q_new = (q - dt/w (v_hi q_up(hi) - v_lo q_up(lo))) / (1 - dt/w (v_hi - v_lo)),
-// the quotient taken as a product with the Newton reciprocal of the denominator.
-__device__ __forceinline__ double vof_step(const GridDev& g, const double* __restrict__ q,
-                                           const double* __restrict__ vel, int axis, int i, int j, int k, double dt,
-                                           double& du) {
-  const size_t plane = (size_t)g.nx * g.ny;
-  int n, bc, f;
-  size_t base, st, fbase, fst;
-  double rw;
-  if (axis == 0) {
-    n = g.nx, bc = g.bcx, f = i, base = (size_t)k * plane + (size_t)j * g.nx, st = 1;
-    fbase = ((size_t)k * g.ny + j) * nface(g.nx, g.bcx), fst = 1, rw = g.rdx;
-  } else if (axis == 1) {
-    n = g.ny, bc = g.bcy, f = j, base = (size_t)k * plane + i, st = g.nx;
-    fbase = (size_t)k * nface(g.ny, g.bcy) * g.nx + i, fst = g.nx, rw = g.rdy;
-  } else {
-    n = g.nz, bc = g.bcz, f = k, base = (size_t)j * g.nx + i, st = plane;
-    fbase = (size_t)j * g.nx + i, fst = plane, rw = __ldg(g.rdz + k);
-  }
-  const int fp = (bc == VOFP_BC_P && f + 1 == n) ? 0 : f + 1;  // the high face of the cell
-  if (!VOFP_IN(base + (size_t)(n - 1) * st, ncells(g), CHK_VOF_LOAD) ||
-      !VOFP_IN(fbase + (size_t)(nface(n, bc) - 1) * fst, nfaces(g, axis), CHK_VOF_LOAD) ||
-      !VOFP_IN(f, n, CHK_VOF_LOAD)) {
-    du = 0.0;
-    return 0.0;
-  }
-  const double vlo = __ldg(vel + fbase + (size_t)f * fst), vhi = __ldg(vel + fbase + (size_t)fp * fst);
-  const double qlo = upwind_value(q, base, st, n, bc, f, vlo);
-  const double qhi = upwind_value(q, base, st, n, bc, f + 1, vhi);
-  const double dtrw = dt * rw, dv = vhi - vlo;
-  du = dv * rw;
-  const double num = fma(-dtrw, fma(vhi, qhi, -vlo * qlo), __ldg(q + base + (size_t)f * st));
-  return num * recip_newton1(fma(-dtrw, dv, 1.0));
-}
-
 // ---- the fused update: one pass marching through the planes -------------------------------------------------
 // A CTA owns a column of kVofTX x kVofTY cells and a run of kVofKC planes [k0, k1).  Marching from plane k0 - 1
 // to k1 (wrapped on a periodic z axis, clamped on a bounded one -- the upwind rule takes the boundary plane
@@ -81,8 +28,11 @@ __device__ __forceinline__ double vof_step(const GridDev& g, const double* __res
 // shared memory) into a ring of three planes, and once C** of m is there, the z step and the correction of Eq.
 // final_corr_2 for plane m - 1, which needs C** of m - 2, m - 1 and m.  C^n, uG, vG, wG are read and C^{n+1}
 // written once per cell (40 bytes) and C*, C** never leave shared memory; the price is the recomputed halo rows
-// and planes (x step x (1 + 2/kVofTY)(1 + 2/kVofKC), y step x (1 + 2/kVofKC)).
-constexpr int kVofTX = 32, kVofTY = 16, kVofKC = 16;
+// and planes (x step x (1 + 2/kVofTY)(1 + 2/kVofKC), y step x (1 + 2/kVofKC)).  Cells whose neighbours hold the same C -- the
+// inside of each phase -- take no FP64 arithmetic: 128^3 droplet 110 us, 218 when every cell did
+// (FP64 pipe 77-84% busy).  Small tiles, for all their halo: the interface makes some tiles long and the others short
+// (32 x 16 x 16 cells 166 us, 16 x 4 126, 8 x 16 131, 4 x 8 125).
+constexpr int kVofTX = 32, kVofTY = 8, kVofKC = 4;
 
 __device__ __forceinline__ int wrap_clamp(int j, int n, int bc) {
   if (j < 0) return bc == VOFP_BC_P ? j + n : 0;
@@ -91,8 +41,11 @@ __device__ __forceinline__ int wrap_clamp(int j, int n, int bc) {
 }
 
 // The implicit one-dimensional step of a cell from its value q, its neighbours' values across the low and
-// high faces (qm, qp) and the two face velocities (as vof_step); sets dv_rw to the velocity difference over
-// the width.
+// high faces (qm, qp) and the two face velocities; sets dv_rw to the velocity difference over the width.  With dt
+// factored out of the fluxes,
+//   q_new = (q - dt/w (v_hi q_up(hi) - v_lo q_up(lo))) / (1 - dt/w (v_hi - v_lo)),
+// q_up the cell the flow comes from (sign bit of the velocity: a zero velocity of either sign gives a zero flux whichever
+// cell is taken), the quotient taken as a product with the Newton reciprocal of the denominator.
 __device__ __forceinline__ double vof_step_local(double qm, double q, double qp, double vlo, double vhi, double rw,
                                                  double dt, double& dv_rw) {
   const double qlo = __double2hiint(vlo) >= 0 ? qm : q;  // upwind across the low face
@@ -101,6 +54,11 @@ __device__ __forceinline__ double vof_step_local(double qm, double q, double qp,
   dv_rw = dv * rw;
   const double num = fma(-dtrw, fma(vhi, qhi, -vlo * qlo), q);
   return num * recip_newton1(fma(-dtrw, dv, 1.0));
+}
+
+// The same where C is the same in the three cells (velocities finite): the step returns it, without arithmetic.
+__device__ __forceinline__ bool vof_flat(double qm, double q, double qp, double vlo, double vhi) {
+  return same_bits(qm, q) && same_value(q, qp) && finite_bits(vlo) && finite_bits(vhi);
 }
 
 static __global__ void __launch_bounds__(kVofTX * kVofTY) k_vof_fused(GridDev g, const double* __restrict__ C,
@@ -121,23 +79,35 @@ static __global__ void __launch_bounds__(kVofTX * kVofTY) k_vof_fused(GridDev g,
   const int nyf = nface(ny, g.bcy);
   // local row r of cs <-> grid row j0 - 1 + r (wrapped or clamped at the ends); rows past ny are unused
   auto row_used = [&](int r) { return j0 - 1 + r <= ny && i < nx; };
-  auto x_step = [&](int k, double* dst) {  // C* of plane k: each thread its row, rows 0 / 1 the halo rows
+  const int nxf = nface(nx, g.bcx);
+  const int im = wrap_clamp(i - 1, nx, g.bcx), iq = wrap_clamp(i + 1, nx, g.bcx);
+  const int ip = (g.bcx == VOFP_BC_P && i + 1 == nx) ? 0 : i + 1;  // the high x face
+  const int jp = (g.bcy == VOFP_BC_P && j + 1 == ny) ? 0 : j + 1;  // the high y face
+  auto x_cell = [&](int k, int row) {  // C* of cell (i, row, k)
+    const size_t cb = ((size_t)k * ny + row) * nx, ub = ((size_t)k * ny + row) * nxf;
+    if (!VOFP_IN(cb + nx - 1, plane * nz, CHK_VOF_LOAD) || !VOFP_IN(ub + nxf - 1, nfaces(g, 0), CHK_VOF_LOAD)) return 0.0;
+    const double vlo = __ldg(uG + ub + i), vhi = __ldg(uG + ub + ip);
+    const double qm = __ldg(C + cb + im), q = __ldg(C + cb + i), qp = __ldg(C + cb + iq);
+    if (vof_flat(qm, q, qp, vlo, vhi)) return q;
     double du;
-    if (row_used(ty + 1)) dst[(ty + 1) * kVofTX + tx] = vof_step(g, C, uG, 0, i, wrap_clamp(j, ny, g.bcy), k, dt, du);
+    return vof_step_local(qm, q, qp, vlo, vhi, g.rdx, dt, du);
+  };
+  auto x_step = [&](int k, double* dst) {  // C* of plane k: each thread its row, rows 0 / 1 the halo rows
+    if (row_used(ty + 1)) dst[(ty + 1) * kVofTX + tx] = x_cell(k, wrap_clamp(j, ny, g.bcy));
     if (ty < 2) {
       const int r = ty == 0 ? 0 : kVofTY + 1;
-      if (row_used(r)) dst[r * kVofTX + tx] = vof_step(g, C, uG, 0, i, wrap_clamp(j0 - 1 + r, ny, g.bcy), k, dt, du);
+      if (row_used(r)) dst[r * kVofTX + tx] = x_cell(k, wrap_clamp(j0 - 1 + r, ny, g.bcy));
     }
   };
   auto y_step = [&](int k, const double* src, double* dst) {  // C** of plane k from C* in shared memory
     if (!act) return;
-    const int jp = (g.bcy == VOFP_BC_P && j + 1 == ny) ? 0 : j + 1;
     const size_t vb = (size_t)k * nyf * nx + i;
     const double vlo = ldg_in(vG, vb + (size_t)j * nx, nfaces(g, 1), CHK_VOF_LOAD);
     const double vhi = ldg_in(vG, vb + (size_t)jp * nx, nfaces(g, 1), CHK_VOF_LOAD);
-    double dv;
-    dst[ty * kVofTX + tx] = vof_step_local(src[ty * kVofTX + tx], src[(ty + 1) * kVofTX + tx],
-                                           src[(ty + 2) * kVofTX + tx], vlo, vhi, g.rdy, dt, dv);
+    const double qm = src[ty * kVofTX + tx], q = src[(ty + 1) * kVofTX + tx], qp = src[(ty + 2) * kVofTX + tx];
+    double v = q, dv;
+    if (!vof_flat(qm, q, qp, vlo, vhi)) v = vof_step_local(qm, q, qp, vlo, vhi, g.rdy, dt, dv);
+    dst[ty * kVofTX + tx] = v;
   };
   // z step and correction of plane k from C** of planes k - 1, k, k + 1 and C* of plane k
   auto finish = [&](int k, const double* qm, const double* q, const double* qp, const double* c1) {
@@ -147,20 +117,22 @@ static __global__ void __launch_bounds__(kVofTX * kVofTY) k_vof_fused(GridDev g,
     const int kp = (g.bcz == VOFP_BC_P && k + 1 == nz) ? 0 : k + 1;
     const double wlo = ldg_in(wG, fb + (size_t)k * plane, nfaces(g, 2), CHK_VOF_LOAD);
     const double whi = ldg_in(wG, fb + (size_t)kp * plane, nfaces(g, 2), CHK_VOF_LOAD);
-    double dw;
-    const double c3 = vof_step_local(qm[o], q[o], qp[o], wlo, whi, __ldg(g.rdz + k), dt, dw);
-    const int nxf = nface(nx, g.bcx);
-    const int ip = (g.bcx == VOFP_BC_P && i + 1 == nx) ? 0 : i + 1;
-    const size_t ub = ((size_t)k * ny + j) * nxf;
-    const double du =
-        (ldg_in(uG, ub + ip, nfaces(g, 0), CHK_VOF_LOAD) - ldg_in(uG, ub + i, nfaces(g, 0), CHK_VOF_LOAD)) * g.rdx;
-    const int jp = (g.bcy == VOFP_BC_P && j + 1 == ny) ? 0 : j + 1;
-    const size_t vb = (size_t)k * nyf * nx + i;
-    const double dv = (ldg_in(vG, vb + (size_t)jp * nx, nfaces(g, 1), CHK_VOF_LOAD) -
-                       ldg_in(vG, vb + (size_t)j * nx, nfaces(g, 1), CHK_VOF_LOAD)) * g.rdy;
-    const double F = fma(c1[(ty + 1) * kVofTX + tx], du, fma(q[o], dv, c3 * dw));
-    if (VOFP_IN((size_t)k * plane + fb, plane * nz, CHK_CELL_STORE))
-      out[(size_t)k * plane + fb] = fma(-dt, F, c3) * recip_newton1(fma(-dt, du + dv + dw, 1.0));
+    const double cs = c1[(ty + 1) * kVofTX + tx], css = q[o];
+    double v = css;
+    // (all three steps returned C: so does the correction, C (1 - dt div uG) / (1 - dt div uG))
+    if (!(vof_flat(qm[o], css, qp[o], wlo, whi) && same_bits(cs, css))) {
+      double dw;
+      const double c3 = vof_step_local(qm[o], css, qp[o], wlo, whi, __ldg(g.rdz + k), dt, dw);
+      const size_t ub = ((size_t)k * ny + j) * nxf;
+      const double du =
+          (ldg_in(uG, ub + ip, nfaces(g, 0), CHK_VOF_LOAD) - ldg_in(uG, ub + i, nfaces(g, 0), CHK_VOF_LOAD)) * g.rdx;
+      const size_t vb = (size_t)k * nyf * nx + i;
+      const double dv = (ldg_in(vG, vb + (size_t)jp * nx, nfaces(g, 1), CHK_VOF_LOAD) -
+                         ldg_in(vG, vb + (size_t)j * nx, nfaces(g, 1), CHK_VOF_LOAD)) * g.rdy;
+      const double F = fma(cs, du, fma(css, dv, c3 * dw));
+      v = fma(-dt, F, c3) * recip_newton1(fma(-dt, du + dv + dw, 1.0));
+    }
+    if (VOFP_IN((size_t)k * plane + fb, plane * nz, CHK_CELL_STORE)) out[(size_t)k * plane + fb] = v;
   };
   for (int m = k0 - 1; m <= k1; ++m) {
     const int s = m - (k0 - 1);  // march step: ring slots s & 1 (C*) and s % 3 (C**)
