@@ -599,6 +599,84 @@ __device__ void zscan_system(const ZArgs& a, TS* col, size_t plane, const TT* F,
   if (bad) atomicOr(&a.info->nonfinite, 1u);
 }
 
+// The same system with every lane's rows (at most R) and factors in registers: each is read once, all reads in flight
+// together.  The low-mode tables only (factors (c'_k, m_k), FP64); a row past the lane's own passes values through.  A 128^3
+// FP32-pair solve's low modes: 12.4 us, 17 us when each of the four sweeps read its rows from memory again.
+template <typename TS, int R>
+__device__ __forceinline__ void zlow_registers(const ZArgs& a, TS* col, size_t plane, const double2* F, size_t fs,
+                                               bool sing, int lane) {
+  const int nz = a.nz, R0 = (nz + 31) >> 5, k0 = lane * R0, kb = sing ? 1 : 0;
+  double al[R], be[R], g[R], wz[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int k = min(k0 + q, nz - 1);
+    const double2 f = __ldg(F + (size_t)k * fs);
+    be[q] = (double)col[(size_t)k * plane];
+    wz[q] = sing ? __ldg(a.dz + k) : 0.0;
+    al[q] = __ldg(a.za + k);
+    g[q] = f.x;
+    al[q] *= -f.y;
+    if (!(q < R0 && k0 + q < nz)) wz[q] = 0.0;
+  }
+  double defect = 0.0;
+  if (sing) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < R; ++q) s = fma(wz[q], be[q], s);
+    defect = warp_sum(s) / a.lz;
+    if (lane == 0 && a.info) a.info->compat_defect = defect * a.scale;
+  }
+  double A = 1.0, B = 0.0;
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int k = k0 + q;
+    const bool own = q < R0 && k < nz && k >= kb;
+    const double m = __ldg(F + (size_t)min(k, nz - 1) * fs).y;
+    be[q] = own ? (be[q] - defect) * (a.scale * m) : 0.0;
+    al[q] = own ? (k > kb ? al[q] : 0.0) : 1.0;
+    g[q] = own ? -g[q] : 1.0;
+    B = fma(al[q], B, be[q]);
+    A *= al[q];
+  }
+  affine_scan_up(A, B, lane);
+  double d = shfl_up_t(B, 1);
+  if (lane == 0) d = 0.0;
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    d = fma(al[q], d, be[q]);
+    be[q] = q < R0 && k0 + q < nz && k0 + q >= kb ? d : 0.0;
+  }
+  A = 1.0;
+  B = 0.0;
+#pragma unroll
+  for (int q = R - 1; q >= 0; --q) {
+    B = fma(g[q], B, be[q]);
+    A *= g[q];
+  }
+  affine_scan_down(A, B, lane);
+  double x = shfl_down_t(B, 1);
+  if (lane == 31) x = 0.0;
+  double ms = 0.0;
+#pragma unroll
+  for (int q = R - 1; q >= 0; --q) {
+    x = fma(g[q], x, be[q]);
+    be[q] = k0 + q >= kb ? x : 0.0;
+    ms = fma(wz[q], be[q], ms);
+  }
+  const double mean = sing ? warp_sum(ms) / a.lz : 0.0;
+  bool bad = false;
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int k = k0 + q;
+    if (q < R0 && k < nz) {
+      const double v = be[q] - mean;
+      col[(size_t)k * plane] = (TS)v;
+      if (a.info) bad |= !isfinite(v);
+    }
+  }
+  if (bad) atomicOr(&a.info->nonfinite, 1u);
+}
+
 // Refinement plans: the low-eigenvalue systems (listed at plan time) in FP64, one warp each; factors k-major
 // (tab[k * nlow + t]), forward values in `scratch` ([nz][nlow]).
 template <typename TS>
@@ -608,8 +686,12 @@ __device__ __forceinline__ void zlow_scan_system(const ZArgs& a, int2 md, int t,
   TS* col = reinterpret_cast<TS*>(a.S) + (size_t)md.y * a.nx + md.x;
   if (!VOFP_IN((size_t)md.y * a.nx + md.x, (size_t)a.nx * a.ny, CHK_Z_COLUMN) || !VOFP_IN(md.x, a.nx, CHK_Z_COLUMN))
     return;  // (uniform per warp)
-  zscan_system<double, TS, double2>(a, col, (size_t)a.nx * a.ny, tab + t, (size_t)nlow, scratch + t, (size_t)nlow,
-                                    a.za, a.singular && md.x == 0 && md.y == 0, lane);
+  const size_t plane = (size_t)a.nx * a.ny;
+  const bool sing = a.singular && md.x == 0 && md.y == 0;
+  if (a.nz <= 128) zlow_registers<TS, 4>(a, col, plane, tab + t, (size_t)nlow, sing, lane);
+  else if (a.nz <= 256) zlow_registers<TS, 8>(a, col, plane, tab + t, (size_t)nlow, sing, lane);
+  else
+    zscan_system<double, TS, double2>(a, col, plane, tab + t, (size_t)nlow, scratch + t, (size_t)nlow, a.za, sing, lane);
 }
 
 template <typename TS>
@@ -624,135 +706,121 @@ static __global__ void __launch_bounds__(128) k_zlow_scan(ZArgs a, const int2* _
 // ---- small grids: systems staged in shared memory -----------------------------------------------------
 // With few systems (nx * ny small) one thread per system leaves most of each SM idle, and an FP64 recurrence
 // is then bound by its 64-cycle dependent latency.  This kernel stages a tile of 32 systems ([nz][32]) in
-// shared memory with all 128 threads, computing alpha_k, beta_k (scaled) and c'_k on the way in; warp 0 runs
-// the two one-multiply-add recurrences from shared memory; warp 1 solves the pinned mean mode (if it is in
-// the tile) by affine scans; all threads store the tile.  Shared memory: nz * 32 * 3 values + nz scratch.
+// shared memory with all 128 threads, as beta_k = s m_k r_k; warp 0 runs the two one-multiply-add recurrences over it, with
+// alpha_k and c'_k read from the factor table 16 rows ahead (a register ring: 16 x 64 cycles cover the reads from L2);
+// warp 1 solves the pinned mean mode (if it is in the tile) by affine scans; all threads store the tile.  With one value a
+// cell in shared memory, 34 KB at 128 rows, all tiles of a 128^3 grid are on the SMs at once and their chains
+// overlap: 32 us; with alpha_k and c'_k staged too (102 KB, two blocks per SM) 48 us.
 constexpr int kZStagedTI = 32;
-template <typename T>
-struct Pair {
-  T x, y;
-};
-inline size_t ztab_staged_smem(int nz, size_t elem) { return (size_t)nz * (3 * kZStagedTI + 1) * elem; }
+inline size_t ztab_staged_smem(int nz, size_t elem) { return (size_t)nz * (kZStagedTI + 1) * elem; }
 // Staged kernel for FP64 / FP32-pair arithmetic when the grid has fewer than 152 * 256 systems (too few to
 // hide the recurrences' latency one thread each) and the tile fits in shared memory.
 inline bool ztab_use_staged(int nx, int ny, int nz, size_t elem) {
   return (size_t)nx * ny < (size_t)152 * 256 && ztab_staged_smem(nz, elem) <= 200 * 1024;
 }
 
+// Both recurrences of one column yc (stride TI) of the tile; F: its factors at stride ts.
+template <typename T, typename TT, int TI>
+__device__ __forceinline__ void ztab_chain(T* yc, const TT* F, size_t ts, int nz) {
+  constexpr int UA = 16, UB = 4;  // rows ahead in the table (L2) and in the tile
+  T fa[UA], yb[UB];
+#pragma unroll
+  for (int u = 0; u < UA; ++u) fa[u] = F[(size_t)min(u, nz - 1) * ts].al;
+#pragma unroll
+  for (int u = 0; u < UB; ++u) yb[u] = yc[min(u, nz - 1) * TI];
+  T v = (T)0;
+  int k = 0;
+  for (; k + UA <= nz; k += UA) {
+#pragma unroll
+    for (int u = 0; u < UA; ++u) {
+      const T al = fa[u], be = yb[u % UB];
+      fa[u] = F[(size_t)min(k + u + UA, nz - 1) * ts].al;
+      yb[u % UB] = yc[min(k + u + UB, nz - 1) * TI];
+      v = fma_t(al, v, be);
+      yc[(k + u) * TI] = v;
+    }
+  }
+  for (; k < nz; ++k) {
+    v = fma_t(F[(size_t)k * ts].al, v, yc[k * TI]);
+    yc[k * TI] = v;
+  }
+  // back from row nz - 2 (row nz - 1 holds its solution)
+#pragma unroll
+  for (int u = 0; u < UA; ++u) fa[u] = F[(size_t)max(nz - 2 - u, 0) * ts].c;
+#pragma unroll
+  for (int u = 0; u < UB; ++u) yb[u] = yc[max(nz - 2 - u, 0) * TI];
+  k = nz - 2;
+  for (; k >= UA - 1; k -= UA) {
+#pragma unroll
+    for (int u = 0; u < UA; ++u) {
+      const T c = fa[u], d = yb[u % UB];
+      fa[u] = F[(size_t)max(k - u - UA, 0) * ts].c;
+      yb[u % UB] = yc[max(k - u - UB, 0) * TI];
+      v = fma_t(-c, v, d);
+      yc[(k - u) * TI] = v;
+    }
+  }
+  for (; k >= 0; --k) {
+    v = fma_t(-F[(size_t)k * ts].c, v, yc[k * TI]);
+    yc[k * TI] = v;
+  }
+}
+
 template <typename T, typename TT>
-static __global__ void __launch_bounds__(128) k_ztab_staged(ZArgs a, ZTabArgs zt) {
+static __global__ void __launch_bounds__(128, 5) k_ztab_staged(ZArgs a, ZTabArgs zt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr int TI = kZStagedTI;
   const int nz = a.nz;
   const int i0 = blockIdx.x * TI, j = blockIdx.y;
-  Pair<T>* ab = reinterpret_cast<Pair<T>*>(smem_raw);  // [nz][TI] (alpha_k, beta_k), then d_k / x_k in .y
-  T* cp = reinterpret_cast<T*>(ab + (size_t)nz * TI);  // [nz][TI] c'_k
-  T* scr = cp + (size_t)nz * TI;                        // [nz] pinned-mode scratch
+  T* yv = reinterpret_cast<T*>(smem_raw);  // [nz][TI] beta_k, then d_k, then x_k
+  T* scr = yv + (size_t)nz * TI;           // [nz] pinned-mode scratch
   const size_t plane = (size_t)a.nx * a.ny;
   T* S = reinterpret_cast<T*>(a.S) + (size_t)j * a.nx + i0;
   const TT* F = reinterpret_cast<const TT*>(zt.tab) + (size_t)distinct_index(j, zt.bcy) * zt.Ux;
   const size_t ts = (size_t)zt.Ux * zt.Uy;
   const T* za = reinterpret_cast<const T*>(zt.za);
-  const T sc = (T)a.scale;
   const int cut = zt.lowcut ? __ldg(zt.lowcut + j) : 0;
   const bool sing_here = a.singular && j == 0 && i0 == 0;  // the pinned mode is column 0 of this tile
   const int ncol = a.nx - i0 < TI ? a.nx - i0 : TI;
   if (!VOFP_IN(i0, a.nx, CHK_Z_COLUMN) || !VOFP_IN((size_t)j * a.nx + i0 + ncol - 1, plane, CHK_Z_COLUMN) ||
       !VOFP_IN((size_t)distinct_index(j, zt.bcy) * zt.Ux + distinct_index(i0 + ncol - 1, zt.bcx), ts, CHK_Z_TABLE))
     return;  // (uniform per block)
-  // tile load: eight rows per thread in flight (all loads issued before any is used)
-  constexpr int UL = 8;
-  for (int t0 = threadIdx.x; t0 < nz * TI; t0 += UL * blockDim.x) {
-    T rv[UL];
-    TT fv[UL];
+  // lane c of every warp on column c of the tile, warp w on rows w, w + 4, ... for the load and the store
+  const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
+  const bool live = c < ncol && i0 + c >= cut && !(sing_here && c == 0);
+  const TT* Fl = F + (c < ncol ? distinct_index(i0 + c, zt.bcx) : 0);
+  if (live) {
+    constexpr int UL = 8;  // rows in flight
+    for (int kb = w; kb < nz; kb += 4 * UL) {
+      T rv[UL], mv[UL];
 #pragma unroll
-    for (int u = 0; u < UL; ++u) {
-      const int t = t0 + u * blockDim.x;
-      const int k = t / TI, c = t - k * TI;
-      if (t < nz * TI && c < ncol && i0 + c >= cut) {
-        fv[u] = F[k * ts + distinct_index(i0 + c, zt.bcx)];
-        rv[u] = S[k * plane + c];
+      for (int u = 0; u < UL; ++u) {
+        const int k = min(kb + 4 * u, nz - 1);
+        mv[u] = Fl[(size_t)k * ts].ms;
+        rv[u] = S[(size_t)k * plane + c];
       }
-    }
 #pragma unroll
-    for (int u = 0; u < UL; ++u) {
-      const int t = t0 + u * blockDim.x;
-      const int k = t / TI, c = t - k * TI;
-      if (t < nz * TI && c < ncol && i0 + c >= cut) {
-        Pair<T> v;
-        v.x = fv[u].al;
-        v.y = rv[u] * fv[u].ms;
-        ab[t] = v;
-        cp[t] = fv[u].c;
+      for (int u = 0; u < UL; ++u) {
+        const T be = rv[u] * mv[u];
+        if (kb + 4 * u < nz) yv[(kb + 4 * u) * TI + c] = be;
       }
     }
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) {
-    const int c = lane, i = i0 + c;
-    if (c < ncol && i >= cut && !(sing_here && c == 0)) {
-      // the shared-memory operands of rows k + 1 .. k + 8 are read before row k is used (a register ring),
-      // so each row costs one dependent multiply-add and no load latency
-      constexpr int U = 8;
-      Pair<T> rb[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (u < nz) rb[u] = ab[u * TI + c];
-      T d = (T)0;
-      for (int k0 = 0; k0 < nz; k0 += U) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int k = k0 + u;
-          if (k < nz) {
-            const Pair<T> v = rb[u];
-            if (k + U < nz) rb[u] = ab[(k + U) * TI + c];
-            d = fma_t(v.x, d, v.y);
-            ab[k * TI + c].y = d;
-          }
-        }
-      }
-      T x = d;
-      T db[U], cb[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = nz - 2 - u;
-        if (k >= 0) {
-          db[u] = ab[k * TI + c].y;
-          cb[u] = cp[k * TI + c];
-        }
-      }
-      for (int k0 = nz - 2; k0 >= 0; k0 -= U) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int k = k0 - u;
-          if (k >= 0) {
-            const T dk = db[u], ck = cb[u];
-            if (k - U >= 0) {
-              db[u] = ab[(k - U) * TI + c].y;
-              cb[u] = cp[(k - U) * TI + c];
-            }
-            x = fma_t(-ck, x, dk);
-            ab[k * TI + c].y = x;
-          }
-        }
-      }
-    }
-  } else if (warp == 1 && sing_here && cut == 0) {
-    zscan_system<T, T, TT>(a, S, plane, F, ts, scr, 1, za, true, lane);
+  if (w == 0) {
+    if (live) ztab_chain<T, TT, TI>(yv + c, Fl, ts, nz);
+  } else if (w == 1 && sing_here && cut == 0) {
+    zscan_system<T, T, TT>(a, S, plane, F, ts, scr, 1, za, true, c);
   }
   __syncthreads();
   bool bad = false;
-  for (int t = threadIdx.x; t < nz * TI; t += blockDim.x) {
-    const int k = t / TI, c = t - k * TI;
-    const int i = i0 + c;
-    if (c < ncol && i >= cut && !(sing_here && c == 0)) {
-      const T x = ab[t].y;
-      S[k * plane + c] = x;
+  if (live)
+    for (int k = w; k < nz; k += 4) {
+      const T x = yv[k * TI + c];
+      S[(size_t)k * plane + c] = x;
       if (a.info) bad |= !isfinite((double)x);
     }
-  }
   if (bad) atomicOr(&a.info->nonfinite, 1u);
 }
 
