@@ -307,22 +307,42 @@ struct VdArgs {
   double rho2;
   double dt;
   double dt_over_rho0;
+  double cc[2];         // dt (1/rho - 1/rho0) where C = 0, C = 1
   double* u;
   double* v;
   double* w;
 };
+// Inside a phase (C exactly 0, or 1, on both sides; an integer test) the coefficient is that phase's constant cc[0 / 1]; where
+// it is zero -- rho0 is the lighter phase's density -- nothing is read but p and C (a pressure that is not finite is left to
+// the arithmetic) and the velocity stays.  128^3 droplet: 86 us, 171 with some 14 FP64 operations on every face.
+__device__ __forceinline__ bool ordinary(double a) { return (__double2hiint(a) & 0x7ff00000) < 0x7f000000; }
 template <int AXIS>
 __device__ __forceinline__ void vd_face(const VdArgs& a, int i, int j, int k) {
   const GridDev& g = a.g;
   FaceRef r;
   if (!corner_face<AXIS>(g, i, j, k, r) || r.e < 0) return;  // (N face: no flux)
-  double d = face_diff(a.pn, r);
-  if (a.pm) d = fma(a.opr, d, -a.r * face_diff(a.pm, r));  // the difference of p_hat
+  const double cl = __ldg(a.C + r.lo), ch = __ldg(a.C + r.hi);
+  double ph = __ldg(a.pn + r.hi), pl = __ldg(a.pn + r.lo), mh = 0.0, ml = 0.0;
+  if (a.pm) {
+    mh = __ldg(a.pm + r.hi);
+    ml = __ldg(a.pm + r.lo);
+  }
+  const bool gas = ((__double_as_longlong(cl) | __double_as_longlong(ch)) << 1) == 0;
+  const bool pure = gas || (same_bits(cl, 1.0) && same_bits(ch, 1.0));
+  const double cc = a.cc[gas ? 0 : 1];
+  if (pure && (__double_as_longlong(cc) << 1) == 0 && ordinary(ph) && ordinary(pl) && ordinary(mh) && ordinary(ml)) return;
+  if (r.e == 2) ph = mh = 0.0;  // (the ghost's sign at a D end, as face_diff)
+  if (r.e == 1) pl = ml = 0.0;
+  double d = one_path(ph) - one_path(pl);
+  if (a.pm) d = fma(a.opr, d, -a.r * (one_path(mh) - one_path(ml)));  // the difference of p_hat
   const double h = face_rdist<AXIS>(g, k, r.e);  // 1 / distance between the values differenced
-  const double rho_f = fma(a.half_drho, __ldg(a.C + r.lo) + __ldg(a.C + r.hi), a.rho2);
-  const double c = h * fma(a.dt, recip_newton(rho_f), -a.dt_over_rho0);  // dt (1/rho_f - 1/rho0) / distance
+  double c = cc;
+  if (!pure) {
+    const double rho_f = fma(a.half_drho, cl + ch, a.rho2);
+    c = fma(a.dt, recip_newton(rho_f), -a.dt_over_rho0);  // dt (1/rho_f - 1/rho0)
+  }
   double* F = AXIS == 0 ? a.u : (AXIS == 1 ? a.v : a.w);
-  F[r.off] = fma(-c, d, F[r.off]);
+  F[r.off] = fma(-(h * one_path(c)), d, F[r.off]);
 }
 static __global__ void __launch_bounds__(kCornerThreads) k_vd_predict(VdArgs a) {
   const int i = blockIdx.x * 32 + (threadIdx.x & 31), k = blockIdx.z;

@@ -500,6 +500,8 @@ extern "C" int vofp_project_vd(vofp_plan* pl, double* u, double* v, double* w, c
   va.rho2 = rho2;
   va.dt = dt;
   va.dt_over_rho0 = dt / rho0;
+  va.cc[0] = dt / rho2 - dt / rho0;
+  va.cc[1] = dt / rho1 - dt / rho0;
   va.u = u;
   va.v = v;
   va.w = w;
