@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xfwd_fx(const
   __shared__ double red[32];
   __shared__ int emax[8], kout[8], lk[16], lj[16];
   __shared__ unsigned l1[8];
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr bool CT = LGN > 0;
   const int n = CT ? 1 << LGN : f.fd.n, lgB = CT ? fx_ct_lgB(LGN) : f.lgB, B = 1 << lgB;
   const int st = CT ? B + 1 : f.st;
@@ -910,19 +910,15 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xfwd_fx(const
     }
   }
   if (stats) {
-    if (!f64) {
-      acc_abs = accf_abs;
-      acc_sq = accf_sq;
-    }
     if (a.info || a.abs_out) {
-      const double s1 = block_sum(acc_abs, red);
+      const double s1 = f64 ? block_sum(acc_abs, red) : block_sum(accf_abs, red);
       if (threadIdx.x == 0 && s1 != 0) {
         if (a.info) atomicAdd(&a.info->abs_sum, s1);
         if (a.abs_out) atomicAdd(a.abs_out, s1);
       }
     }
     if (a.sq_out) {
-      const double s2 = block_sum(acc_sq, red);
+      const double s2 = f64 ? block_sum(acc_sq, red) : block_sum(accf_sq, red);
       if (threadIdx.x == 0 && s2 != 0) atomicAdd(a.sq_out, s2);
     }
     if (a.fv_out) {
@@ -967,7 +963,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_ypass_fx(cons
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int emax[8];
   __shared__ unsigned l1[8];
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr bool CT = LGN > 0;
   const int n = CT ? 1 << LGN : f.fd.n, lgB = CT ? fx_ct_lgB(LGN) : f.lgB, B = 1 << lgB;
   const int st = CT ? B : f.st;
@@ -1028,7 +1024,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xinv_fx(const
   __shared__ double red[32];
   __shared__ int emax[8], kout[8];
   __shared__ unsigned l1[8];
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr bool CT = LGN > 0;
   const int n = CT ? 1 << LGN : f.fd.n, lgB = CT ? fx_ct_lgB(LGN) : f.lgB, B = 1 << lgB;
   const int st = CT ? B + 1 : f.st;

@@ -129,6 +129,23 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
+// The same of FP32 partial sums, as FP32 pairs within a warp (32 floats add up exactly in their 48 bits but for the
+// extremes): five shuffled FP64 additions a thread and sum were two FP64 operations a cell.
+__device__ __forceinline__ double block_sum(float v, double* red) {
+  ff p(v, 0.0f);
+  for (int o = 16; o > 0; o >>= 1)
+    p += ff(__shfl_down_sync(0xffffffffu, p.hi, o), __shfl_down_sync(0xffffffffu, p.lo, o));
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  if (lane == 0) red[wid] = (double)p;
+  __syncthreads();
+  double s = 0;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
+  }
+  return s;
+}
+
 // Item t of a block's (line pair, sample) loop: pair t / n, sample t % n -- by shift and mask for a
 // power-of-two n (lgn >= 0), else by division.
 __device__ __forceinline__ void split_item(int t, int n, int lgn, int& pb, int& i) {
@@ -152,7 +169,7 @@ __device__ __forceinline__ void xfwd_block(const XArgs& a, int bx, unsigned char
   const int PB = a.pb;
   const int ld = fft_span(a.fd, a.blu);
   C* b1 = b0 + PB * ld;
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const long nlines = (long)a.g.ny * a.g.nz;
   const long pair0 = (long)bx * PB;
   const int bc = a.g.bcx;
@@ -219,19 +236,15 @@ __device__ __forceinline__ void xfwd_block(const XArgs& a, int bx, unsigned char
     }
     b0[pb * ld + idx] = cmk<C>(neg_if(fa, fl), neg_if(fb, fl));
   }
-  if (!f64) {
-    acc_abs = accf_abs;
-    acc_sq = accf_sq;
-  }
   if (a.info || a.abs_out) {
-    const double s1 = block_sum(acc_abs, red);
+    const double s1 = f64 ? block_sum(acc_abs, red) : block_sum(accf_abs, red);
     if (threadIdx.x == 0 && s1 != 0) {
       if (a.info) atomicAdd(&a.info->abs_sum, s1);
       if (a.abs_out) atomicAdd(a.abs_out, s1);
     }
   }
   if (a.sq_out) {
-    const double s2 = block_sum(acc_sq, red);
+    const double s2 = f64 ? block_sum(acc_sq, red) : block_sum(accf_sq, red);
     if (threadIdx.x == 0 && s2 != 0) atomicAdd(a.sq_out, s2);
   }
   if (a.fv_out) {
@@ -284,7 +297,7 @@ struct YArgs {
 template <typename T, typename C, bool INV>
 __device__ __forceinline__ void ypass_block(const YArgs& a, int bx, int by, unsigned char* smem_raw) {
   typedef decltype(C::x) R;
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int n = a.ny;
   const int B = a.tx >> 1;
   C* b0 = reinterpret_cast<C*>(smem_raw);
@@ -410,7 +423,7 @@ struct XInvArgs {
 template <typename T, typename C>
 __device__ __forceinline__ void xinv_block(const XInvArgs& a, int bx, unsigned char* smem_raw, double* red) {
   typedef decltype(C::x) R;
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int n = a.nx;
   const int PB = a.pb;
   const int ld = fft_span(a.fd, a.blu);
@@ -508,16 +521,13 @@ __device__ __forceinline__ void xinv_block(const XInvArgs& a, int bx, unsigned c
       }
     }
   }
-  if (!f64) {
-    acc = (double)accm;
-    acc2 = acc2f;
-  }
+  if (!f64) acc = (double)accm;
   if (a.mean_out) {
     const double s = block_sum(acc, red);
     if (threadIdx.x == 0 && s != 0) atomicAdd(a.mean_out, s);
   }
   if (a.d2_out) {
-    const double s = block_sum(acc2, red);
+    const double s = f64 ? block_sum(acc2, red) : block_sum(acc2f, red);
     if (threadIdx.x == 0 && s != 0) atomicAdd(a.d2_out, s);
   }
 }

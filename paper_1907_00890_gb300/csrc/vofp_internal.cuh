@@ -113,6 +113,14 @@ __device__ __forceinline__ bool launch_skipped(const double* conv, int j, double
   return refine_done(conv, j, tol2);
 }
 
+// The same by one thread for the whole block (every thread calls it): the test is some ten FP64 operations, which every
+// thread of a launch would queue on the FP64 pipe.
+__device__ __forceinline__ bool block_skipped(const double* conv, int j, double tol2) {
+  if (j <= -2) return true;
+  if (!conv || j <= 0) return false;
+  return __syncthreads_or(threadIdx.x == 0 && refine_done(conv, j, tol2));
+}
+
 // Most line pairs per block of an x pass (the plan's default takes at most 16, the tuner at most 32).
 constexpr int kMaxPB = 32;
 

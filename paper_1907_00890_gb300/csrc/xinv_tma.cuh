@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kXTmaThreads) k_xinv_tma(const XTmaArgs a, con
                                                            const __grid_constant__ CUtensorMap tp) {
   typedef typename CplxOf<T>::C C;
   const XInvArgs& x = a.xi;
-  if (launch_skipped(x.skip_conv, x.skip_k, x.tol2)) return;
+  if (block_skipped(x.skip_conv, x.skip_k, x.tol2)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long bar[3];  // the two spectrum tiles, the potential's rows
   __shared__ double red[32];
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kXTmaThreads) k_xinv_tma(const XTmaArgs a, con
     if (threadIdx.x == 0 && s != 0) atomicAdd(x.mean_out, s);
   }
   if (x.d2_out) {
-    const double s = block_sum((double)acc2f, red);
+    const double s = block_sum(acc2f, red);
     if (threadIdx.x == 0 && s != 0) atomicAdd(x.d2_out, s);
   }
 }

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kYTmaThreads) k_ypass_tma(const YTmaArgs a, co
   typedef typename CplxOf<T>::C C;
   constexpr bool CT = LGN > 0;
   const YArgs& y = a.y;
-  if (launch_skipped(y.skip_conv, y.skip_k, y.tol2)) return;
+  if (block_skipped(y.skip_conv, y.skip_k, y.tol2)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long bar[2];
   const int n = CT ? (1 << LGN) : y.ny, lgn = CT ? LGN : 31 - __clz(n);

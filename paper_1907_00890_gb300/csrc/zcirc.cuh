@@ -146,7 +146,7 @@ __device__ void zcirc_singular(const ZArgs& a, TS* col, size_t plane, int lane) 
 template <typename T>
 __device__ __forceinline__ void zcirc_block(const ZArgs& a, const ZCircArgs& z, int bx, int by,
                                             unsigned char* smem_raw) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int TI = z.ti, nz = a.nz, NS = kZCircThreads / TI, L = z.L;
   const int c = threadIdx.x & (TI - 1), sg = threadIdx.x / TI;
   const int i = bx * TI + c, j = by;
@@ -244,7 +244,7 @@ static __global__ void __launch_bounds__(kZCircThreads) k_zcirc(ZArgs a, ZCircAr
 template <typename TS>
 static __global__ void __launch_bounds__(128) k_zcirc_low(ZArgs a, const int2* __restrict__ modes, int nlow,
                                                           const ZCirc<double>* __restrict__ tab, double* scratch) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= nlow) return;  // uniform per warp
   const int2 md = modes[w];

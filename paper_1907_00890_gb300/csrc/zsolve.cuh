@@ -129,7 +129,7 @@ __device__ void solve_column(const ZArgs& a, int iq, int jq, Col<TA> d, Col<TA> 
 // One block: `ti` neighbouring x indices of one y index, staged [nz][ti] in shared memory.
 template <typename TS, typename TA>
 __device__ __forceinline__ void zsolve_block(const ZArgs& a, int bx, int by, unsigned char* smem_raw) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int TI = a.ti, nz = a.nz;
   TA* d = reinterpret_cast<TA*>(smem_raw);
   TA* cp = d + (size_t)nz * TI;
@@ -247,7 +247,7 @@ __device__ __forceinline__ void zlow_system(const ZArgs& a, int2 md, int t, int 
 template <typename TS>
 __global__ void k_zlow64(ZArgs a, const int2* __restrict__ modes, int nlow, const double2* __restrict__ tab,
                          double* scratch) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nlow) return;
   zlow_system<TS>(a, modes[t], t, nlow, tab, scratch);
@@ -422,7 +422,7 @@ __device__ bool ztab_singular(const ZArgs& a, T* col, T* dcol, size_t ds, size_t
 template <typename T, typename TT>
 __device__ __forceinline__ void ztab_block(const ZArgs& a, const ZTabArgs& zt, int smem_d, int bx, int by,
                                            unsigned char* smem_raw) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int TI = blockDim.x, nz = a.nz;
   const int c = threadIdx.x;
   const int i = bx * TI + c, j = by;
@@ -697,7 +697,7 @@ __device__ __forceinline__ void zlow_scan_system(const ZArgs& a, int2 md, int t,
 template <typename TS>
 static __global__ void __launch_bounds__(128) k_zlow_scan(ZArgs a, const int2* __restrict__ modes, int nlow,
                                                           const double2* __restrict__ tab, double* scratch) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= nlow) return;  // uniform per warp
   zlow_scan_system<TS>(a, modes[w], w, nlow, tab, scratch, threadIdx.x & 31);
@@ -769,7 +769,7 @@ __device__ __forceinline__ void ztab_chain(T* yc, const TT* F, size_t ts, int nz
 template <typename T, typename TT>
 static __global__ void __launch_bounds__(128, 5) k_ztab_staged(ZArgs a, ZTabArgs zt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr int TI = kZStagedTI;
   const int nz = a.nz;
   const int i0 = blockIdx.x * TI, j = blockIdx.y;
@@ -861,7 +861,7 @@ inline int ztab_seg_code(int nz, size_t elem) {
 template <typename T, typename TT, bool LEAN>
 __device__ __forceinline__ void ztab_seg_block(const ZArgs& a, const ZTabArgs& zt, int bx, int by,
                                                unsigned char* smem_raw) {
-  if (launch_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
+  if (block_skipped(a.skip_conv, a.skip_k, a.tol2)) return;
   constexpr int TI = kZSegTI, W = kZSegW;
   const int nz = a.nz;
   const int i0 = bx * TI, j = by;
