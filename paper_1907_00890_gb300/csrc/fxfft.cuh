@@ -859,6 +859,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xfwd_fx(const
   const bool stats = a.info || a.sq_out || a.fv_out || a.abs_out;
   constexpr bool f64 = std::is_same<T, double>::value;
   const double fbar = (MODE == RHS_RESID && a.defect_sum) ? *a.defect_sum * a.inv_volume : 0.0;
+  constexpr bool fv = MODE != RHS_RESID;  // (a residual's sum is not asked for: no multiply-add predicated off)
   double acc_abs = 0, acc_sq = 0, acc_fv = 0;
   float accf_abs = 0.0f, accf_sq = 0.0f;
   const int total = n << lgB;
@@ -899,7 +900,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xfwd_fx(const
             const float fs = f32_lead_bits(r);
             accf_abs = fmaf(fabsf(fs), __ldg(a.g.volf + k), accf_abs);
             accf_sq = fmaf(fs, fs, accf_sq);
-            if (a.fv_out) acc_fv = fma(r, __ldg(a.g.vol + k), acc_fv);
+            if (fv && a.fv_out) acc_fv = fma(r, __ldg(a.g.vol + k), acc_fv);
           }
         }
       }
@@ -921,7 +922,7 @@ __global__ void __launch_bounds__(fx_bound(LGN), fx_blocks(LGN)) k_xfwd_fx(const
       const double s2 = f64 ? block_sum(acc_sq, red) : block_sum(accf_sq, red);
       if (threadIdx.x == 0 && s2 != 0) atomicAdd(a.sq_out, s2);
     }
-    if (a.fv_out) {
+    if (fv && a.fv_out) {
       const double s3 = block_sum(acc_fv, red);
       if (threadIdx.x == 0 && s3 != 0) atomicAdd(a.fv_out, s3);
     }

@@ -40,7 +40,7 @@ struct XArgs {
   double* fsave;      // if non-null, the FP64 right-hand side is stored here (mixed path)
   vofp_devinfo* info; // if non-null, accumulate sum |f| V into info->abs_sum
   double* sq_out;     // if non-null, accumulate sum f^2 here
-  double* fv_out;     // if non-null, accumulate sum f V here
+  double* fv_out;     // if non-null, accumulate sum f V here (not RHS_RESID)
   double* abs_out;    // if non-null, accumulate sum |f| V here
   const double* skip_conv;  // mixed refinement: skip when conv[3 + skip_k] <= tol2 conv[0]
   int skip_k;
@@ -187,6 +187,7 @@ __device__ __forceinline__ void xfwd_block(const XArgs& a, int bx, unsigned char
   // in FP64 and accumulate the norms, which feed thresholds only, in FP32
   constexpr bool f64 = std::is_same<T, double>::value;
   const double fbar = (MODE == RHS_RESID && a.defect_sum) ? *a.defect_sum * a.inv_volume : 0.0;
+  constexpr bool fv = MODE != RHS_RESID;  // (a residual's sum is not asked for: no multiply-add predicated off)
   double acc_abs = 0, acc_sq = 0, acc_fv = 0;
   float accf_abs = 0.0f, accf_sq = 0.0f;
   for (int t = threadIdx.x; t < PB * n; t += blockDim.x) {
@@ -212,7 +213,7 @@ __device__ __forceinline__ void xfwd_block(const XArgs& a, int bx, unsigned char
             const float fs = lead(fr);
             accf_abs = fmaf(fabsf(fs), __ldg(a.g.volf + k), accf_abs);
             accf_sq = fmaf(fs, fs, accf_sq);
-            if (a.fv_out) acc_fv = fma(f, __ldg(a.g.vol + k), acc_fv);
+            if (fv && a.fv_out) acc_fv = fma(f, __ldg(a.g.vol + k), acc_fv);
           }
         }
         if (h)
@@ -247,7 +248,7 @@ __device__ __forceinline__ void xfwd_block(const XArgs& a, int bx, unsigned char
     const double s2 = f64 ? block_sum(acc_sq, red) : block_sum(accf_sq, red);
     if (threadIdx.x == 0 && s2 != 0) atomicAdd(a.sq_out, s2);
   }
-  if (a.fv_out) {
+  if (fv && a.fv_out) {
     const double s3 = block_sum(acc_fv, red);
     if (threadIdx.x == 0 && s3 != 0) atomicAdd(a.fv_out, s3);
   }
