@@ -261,7 +261,7 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
   std::vector<double2> tw[2], quart[2];
   std::vector<float2> tw32[2], quart32[2];
   std::vector<cff> twff[2], quartff[2];
-  std::vector<fxtw> twfx[2];  // fixed-point tables (FP64 and FP32-pair plans, lengths without a Bluestein form)
+  std::vector<fxtw> twfx[2];  // fixed-point tables (see fx_takes)
   std::vector<fxq> quartfx[2];
   std::vector<double2> blu[2];  // Bluestein tables (empty when the axis needs none)
   auto to_cff = [](double2 z) {
@@ -300,8 +300,7 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     p->ax[a].n = n;
     p->ax[a].bc = bc[a];
     if (p->ax[a].fd.bm) blu[a] = bluestein_tables(p->ax[a].fd);
-    FxDesc fx;
-    if (o.prec != VOFP_MIXED && fx_desc(p->ax[a].fd, &fx)) {
+    if (o.prec != VOFP_MIXED && fx_takes(p->ax[a].fd, o.prec == VOFP_FF)) {
       twfx[a].resize(n);
       quartfx[a].resize(nq);
       for (int q = 0; q < n; ++q) {
