@@ -990,8 +990,8 @@ def measured_traffic(workload, kernel):
 def algorithmic(kname, n):
     """Algorithmic HBM bytes and FP64 flops of one launch of kernel class ``kname`` on an n-grid.
 
-    Bytes: each compulsory array read or written once (8 B per FP64 value).  Flops: a real-to-real transform
-    of length m counts 2.5 m log2 m per line (half the 5 m log2 m of a complex FFT); the z recurrence with
+    Bytes: each compulsory array read or written once (8 B per FP64 value).  Flops: the transforms count none (they run
+    in 64-bit fixed point on the integer pipe; only right-hand sides are formed in FP64); the z recurrence with
     plan-time factors 6 per point (forward multiply-add and multiply, back multiply-add, output scale);
     stencils their adds and multiplies (a multiply-add counts 2): the velocity correction a difference and a
     multiply-add per face (3, one more product on z faces: 10 per cell), the extension a difference, two face
@@ -1000,19 +1000,15 @@ def algorithmic(kname, n):
     """
     nx, ny, nz = n
     cells = nx * ny * nz
-
-    def lg(m):
-        return math.log2(m) if m > 1 else 0.0
-
     tab = {
-        "x_forward": (16, 2.5 * lg(nx)),
-        "x_forward_div": (32, 8 + 2.5 * lg(nx)),
-        "x_forward_stefan": (24, 18 + 2.5 * lg(nx)),
-        "x_forward_div_stefan": (48, 26 + 2.5 * lg(nx)),
-        "y_forward": (16, 2.5 * lg(ny)),
-        "y_inverse": (16, 2.5 * lg(ny)),
+        "x_forward": (16, 0),
+        "x_forward_div": (32, 8),
+        "x_forward_stefan": (24, 18),
+        "x_forward_div_stefan": (48, 26),
+        "y_forward": (16, 0),
+        "y_inverse": (16, 0),
         "z_tridiag": (16, 6),
-        "x_inverse": (16, 2.5 * lg(nx)),
+        "x_inverse": (16, 0),
         "grad_update": (56, 10),
         "extend_epilogue": (96, 24),
         "stefan_source": (48, 20),
@@ -1077,8 +1073,8 @@ def run_only(args):
 
 
 # kernel function name (as ncu prints it) -> the library's trace class
-_KCLASS = [(r"k_zfactor", None), (r"k_zlow", "z_low_modes"), (r"k_z", "z_tridiag"), (r"k_xinv", "x_inverse"),
-           (r"k_xtc\b", "x_tensor_core"), (r"k_grad", "grad_update"), (r"k_extend_epi", "extend_epilogue"),
+_KCLASS = [(r"k_zfactor|k_zcirc(_low)?_table", None), (r"k_zlow|k_zcirc_low", "z_low_modes"), (r"k_z", "z_tridiag"),
+           (r"k_xinv", "x_inverse"), (r"k_xtc\b", "x_tensor_core"), (r"k_grad", "grad_update"), (r"k_extend_epi", "extend_epilogue"),
            (r"k_geometry", "stefan_source"), (r"k_vd_predict", "vd_predict"), (r"k_vof_fused", "vof_update"),
            (r"k_shift", "gauge_shift")]
 _XMODE = {0: "x_forward", 1: "x_forward_div", 2: "x_forward_stefan", 3: "residual_update", 4: "x_forward_div"}
@@ -1111,9 +1107,10 @@ def kernel_class(name):
     import re
     ta = [re.sub(r"^\(\w+\)", "", t) for t in _template_args(name)]
     if re.search(r"k_xfwd", name) and ta:
-        return _XMODE.get(int(ta[-1])) if ta[-1].isdigit() else None
+        mode = ta[1] if "k_xfwd_fx" in name else ta[-1]  # (fixed point: <type, mode, length>)
+        return _XMODE.get(int(mode)) if mode.isdigit() else None
     if re.search(r"k_ypass", name) and ta:
-        inv = ta[1] if "k_ypass_tma" in name else ta[-1]
+        inv = ta[1] if "k_ypass_tma" in name or "k_ypass_fx" in name else ta[-1]
         return "y_inverse" if inv in ("true", "1") else "y_forward"
     for pat, cls in _KCLASS:
         if re.search(pat, name):
