@@ -25,10 +25,10 @@ __host__ __device__ __forceinline__ int corner_tiles_y(const GridDev& g) {
   return (nface(g.ny, g.bcy) + kCornerRows - 1) / kCornerRows;
 }
 constexpr int kCornerThreads = 512;  // at most
-// Threads per tile: four warps of four rows each; sixteen of one row where the tiles are fewer than two per SM (a 32^3
-// correction took 5 us longer with four).
+// Threads per tile: four warps of four rows each; sixteen of one row while the tiles are fewer than four per SM, all of them
+// resident (a 32^3 correction took 5 us longer with four, the extension of 20 x 20 x 160, 320 tiles, 16.6 us with four, 12.4 with sixteen).
 inline int corner_threads(const GridDev& g) {
-  return (long)corner_tiles_x(g) * corner_tiles_y(g) * nface(g.nz, g.bcz) < 304 ? 512 : 128;
+  return (long)corner_tiles_x(g) * corner_tiles_y(g) * nface(g.nz, g.bcz) < 608 ? 512 : 128;
 }
 inline dim3 corner_grid(const GridDev& g) {
   return dim3((unsigned)corner_tiles_x(g), (unsigned)corner_tiles_y(g), (unsigned)nface(g.nz, g.bcz));

@@ -105,11 +105,25 @@ inline bool fx_desc(const FftDesc& fd, FxDesc* fx) {
 // (122) 50 against 129-148, 151 101 against 150-158, 197 135 against 186-198, 251 172 against 133-162; FP32 pairs at p = 17
 // 26 against 57, 47 (188) 44 against 50, 53 (106) 48 against 62, 61 (122) 52 against 44 (its convolution has a lucky 256
 // points), 79 (158) 66 against 50.
-inline bool fx_takes(const FftDesc& fd, bool ff) {
+// Other lengths on small grids: a pass is one short wave of blocks, bound by the latency of its chain, and that of the
+// fixed-point passes is the longer one.  Measured, one pass, floating point against fixed point: FP64, lengths without a
+// compiled-in kernel, x 48 (110592 cells) 1 : 0.81-1.00, 24 (144000) 0.80-0.95, 96 (221088) 1.11-1.15, y 20 (64000) 0.8, 48
+// (110592) 0.8, 24 (198144) 0.90, 96 (209664) 1.24, but 384 (98304) 2.0; compiled-in 64 (65536) 1.05-1.3; 32, a warp per block: a
+// 32^3 projection 64 -> 53 us, x 61440 cells 0.90-1.02, 173376 0.74-0.96, y 86016 0.91, 326656 1.26.  FP32 pairs, any length: x 48
+// (110592) 0.66-0.73, 64 (336896) 0.83-1.20, 72 (460800) 0.90-1.05, y 96 (61440) 0.7, 192 (380160) 0.96; without a compiled-in
+// kernel, x 80 (512000) 0.78-0.91, 100 (864000) 0.81-0.96, y 96 (864000) 0.73-0.78; 32 x 128 x 128 no slower.
+// `force` (VOFP_FX=1 when the plan is created): fixed point whatever the grid, for comparisons.
+inline bool fx_takes(const FftDesc& fd, bool ff, bool y, long cells, bool force) {
   FxDesc fx;
   for (int s = 0; s < fd.nst; ++s)
     if (fd.radix[s] > (ff ? 53 : 199)) return false;
-  return fx_desc(fd, &fx);
+  if (!fx_desc(fd, &fx)) return false;
+  if (force || fd.bm) return true;
+  const bool pow2 = (fd.n & (fd.n - 1)) == 0;
+  if (ff) return cells >= (pow2 && fd.n >= 32 && fd.n <= 512 ? 480000 : 2000000);
+  if (pow2 && fd.n >= 64 && fd.n <= 512) return true;
+  if (fd.n == 32) return cells <= 48000 || cells >= (y ? 200000 : 480000);
+  return cells >= 200000 || (y && fd.n >= 256);
 }
 
 // ---- scalars ------------------------------------------------------------------------------------------------

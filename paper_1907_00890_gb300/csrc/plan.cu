@@ -262,6 +262,8 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
   std::vector<float2> tw32[2], quart32[2];
   std::vector<cff> twff[2], quartff[2];
   std::vector<fxtw> twfx[2];  // fixed-point tables (see fx_takes)
+  const char* fx_env = getenv("VOFP_FX");
+  const bool fx_force = fx_env && fx_env[0] == '1';
   std::vector<fxq> quartfx[2];
   std::vector<double2> blu[2];  // Bluestein tables (empty when the axis needs none)
   auto to_cff = [](double2 z) {
@@ -300,7 +302,7 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     p->ax[a].n = n;
     p->ax[a].bc = bc[a];
     if (p->ax[a].fd.bm) blu[a] = bluestein_tables(p->ax[a].fd);
-    if (o.prec != VOFP_MIXED && fx_takes(p->ax[a].fd, o.prec == VOFP_FF)) {
+    if (o.prec != VOFP_MIXED && fx_takes(p->ax[a].fd, o.prec == VOFP_FF, a == 1, (long)nx * ny * nz, fx_force)) {
       twfx[a].resize(n);
       quartfx[a].resize(nq);
       for (int q = 0; q < n; ++q) {
