@@ -26,7 +26,8 @@ __host__ __device__ __forceinline__ int corner_tiles_y(const GridDev& g) {
 }
 constexpr int kCornerThreads = 512;  // at most
 // Threads per tile: four warps of four rows each; sixteen of one row while the tiles are fewer than four per SM, all of them
-// resident (a 32^3 correction took 5 us longer with four, the extension of 20 x 20 x 160, 320 tiles, 16.6 us with four, 12.4 with sixteen).
+// resident (a 32^3 correction took 5 us longer with four; the extension of 20 x 20 x 160, 320 tiles: 16.6 us with four, 12.4 with
+// sixteen).
 inline int corner_threads(const GridDev& g) {
   return (long)corner_tiles_x(g) * corner_tiles_y(g) * nface(g.nz, g.bcz) < 608 ? 512 : 128;
 }
@@ -314,7 +315,7 @@ struct VdArgs {
 };
 // Inside a phase (C exactly 0, or 1, on both sides; an integer test) the coefficient is that phase's constant cc[0 / 1]; where
 // it is zero -- rho0 is the lighter phase's density -- nothing is read but p and C (a pressure that is not finite is left to
-// the arithmetic) and the velocity stays.  128^3 droplet: 86 us, 171 with some 14 FP64 operations on every face.
+// the arithmetic) and the velocity stays.  128^3 droplet: 74 us, 171 with some 14 FP64 operations on every face.
 __device__ __forceinline__ bool ordinary(double a) { return (__double2hiint(a) & 0x7ff00000) < 0x7f000000; }
 template <int AXIS>
 __device__ __forceinline__ void vd_face(const VdArgs& a, int i, int j, int k) {
@@ -344,14 +345,17 @@ __device__ __forceinline__ void vd_face(const VdArgs& a, int i, int j, int k) {
   double* F = AXIS == 0 ? a.u : (AXIS == 1 ? a.v : a.w);
   F[r.off] = fma(-(h * one_path(c)), d, F[r.off]);
 }
-static __global__ void __launch_bounds__(kCornerThreads) k_vd_predict(VdArgs a) {
-  const int i = blockIdx.x * 32 + (threadIdx.x & 31), k = blockIdx.z;
-  for (int q = threadIdx.x >> 5; q < kCornerRows; q += blockDim.x >> 5) {
-    const int j = blockIdx.y * kCornerRows + q;
-    vd_face<0>(a, i, j, k);
-    vd_face<1>(a, i, j, k);
-    vd_face<2>(a, i, j, k);
-  }
+// (Lanes run over the corners of a plane row after row: a tile of 32 a row leaves lanes of the FP64 pipe's turns idle where a
+// row is no multiple of 32: 128^3 86 -> 74 us, 20 x 20 x 160 25 -> 14, 34 x 134 x 64 58 -> 30.)
+constexpr int kVdThreads = 128;
+inline dim3 vd_grid(const GridDev& g) {
+  return dim3((unsigned)((nface(g.nx, g.bcx) * nface(g.ny, g.bcy) + kVdThreads - 1) / kVdThreads), (unsigned)nface(g.nz, g.bcz));
+}
+static __global__ void __launch_bounds__(kVdThreads) k_vd_predict(VdArgs a) {
+  const int c = blockIdx.x * kVdThreads + threadIdx.x, fx = nface(a.g.nx, a.g.bcx), j = c / fx, i = c - j * fx, k = blockIdx.y;
+  vd_face<0>(a, i, j, k);
+  vd_face<1>(a, i, j, k);
+  vd_face<2>(a, i, j, k);
 }
 
 }  // namespace vofp

@@ -505,7 +505,7 @@ extern "C" int vofp_project_vd(vofp_plan* pl, double* u, double* v, double* w, c
   va.u = u;
   va.v = v;
   va.w = w;
-  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<corner_grid(va.g), corner_threads(va.g), 0, st>>>(va));
+  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<vd_grid(va.g), kVdThreads, 0, st>>>(va));
   if (cudaGetLastError() != cudaSuccess) return VOFP_ERR_CUDA;
   return vofp_project(pl, u, v, w, src, dt / rho0, p, stream, info);
 }
