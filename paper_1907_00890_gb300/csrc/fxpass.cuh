@@ -40,7 +40,7 @@ static FxXFwd fx_xfwd_mode(int mode) {
 }
 template <typename T>
 static FxXFwd fx_xfwd_kernel(int mode, int lgn) {
-  switch (mode == RHS_DIV_STEFAN ? 0 : lgn) {
+  switch (lgn) {
     case 5: return fx_xfwd_mode<T, 5>(mode);
     case 6: return fx_xfwd_mode<T, 6>(mode);
     case 7: return fx_xfwd_mode<T, 7>(mode);
@@ -90,13 +90,17 @@ void init_fx_attributes() {
   }
 }
 
-// Tables and tile of axis ax for tiles8 tiles of eight lines; false: the axis' length has no fixed-point form.
-static bool fx_tables(const vofp_plan* pl, int ax, long tiles8, int least, FxTables* f) {
+// Tables and tile of axis ax for tiles8 tiles of eight lines, and the kernel for it (*lgn: a compiled-in length, or 0 for the
+// run-time one, which `rt` asks for); false: the axis' length has no fixed-point form.
+static bool fx_tables(const vofp_plan* pl, int ax, long tiles8, int least, bool rt, FxTables* f, int* lgn) {
   const AxisDev& a = pl->ax[ax];
   if (!a.twfx || !fx_desc(a.fd, &f->fd)) return false;
   f->tw = (const fxtw*)a.twfx;
   f->quart = (const fxq*)a.quartfx;
   f->lgB = fx_lgB(a.n, tiles8, least);
+  *lgn = rt ? 0 : fx_lgn(*f);
+  // (the run-time kernels are bound to kFxMaxThreads: eight lines of 512 samples are a compiled-in kernel's tile only)
+  while (fx_threads(a.n, f->lgB) > fx_bound(*lgn)) --f->lgB;
   f->st = (1 << f->lgB) + (ax == 0 ? 1 : 0);
   return true;
 }
@@ -105,11 +109,12 @@ template <typename T>
 bool fx_xfwd(vofp_plan* pl, int mode, const XArgs& xa, cudaStream_t st) {
   FxTables f;
   const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
-  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, &f)) return false;
+  int lgn;
+  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, mode == RHS_DIV_STEFAN, &f, &lgn)) return false;
   const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
   const int kid = mode == RHS_F ? KID_XFWD : (mode == RHS_DIV ? KID_XFWD_DIV : (mode == RHS_RESID ? KID_RESID : KID_XFWD_DIVSTEF));
-  const FxXFwd kern = mode == RHS_STEFAN ? nullptr : fx_xfwd_kernel<T>(mode, fx_lgn(f));
+  const FxXFwd kern = mode == RHS_STEFAN ? nullptr : fx_xfwd_kernel<T>(mode, lgn);
   if (!kern) return false;
   VOFP_LAUNCH(kid, st, (kern<<<grid, th, sm, st>>>(xa, f)));
   return true;
@@ -117,22 +122,24 @@ bool fx_xfwd(vofp_plan* pl, int mode, const XArgs& xa, cudaStream_t st) {
 template <typename T>
 bool fx_ypass(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st) {
   FxTables f;
+  int lgn;
   const int nx = pl->n[0], nz = pl->n[2];
-  if (!fx_tables(pl, 1, (long)((nx + 15) / 16) * nz, 1, &f)) return false;
+  if (!fx_tables(pl, 1, (long)((nx + 15) / 16) * nz, 1, false, &f, &lgn)) return false;
   const dim3 grid((nx + (2 << f.lgB) - 1) / (2 << f.lgB), nz);
   const int th = fx_threads(f.fd.n, f.lgB);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
-  VOFP_LAUNCH(inv ? KID_YINV : KID_YFWD, st, (fx_ypass_kernel<T>(inv, fx_lgn(f))<<<grid, th, sm, st>>>(ya, f)));
+  VOFP_LAUNCH(inv ? KID_YINV : KID_YFWD, st, (fx_ypass_kernel<T>(inv, lgn)<<<grid, th, sm, st>>>(ya, f)));
   return true;
 }
 template <typename T>
 bool fx_xinv(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
   FxTables f;
   const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
-  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, &f)) return false;
+  int lgn;
+  if (!fx_tables(pl, 0, (npairs + 7) / 8, 0, false, &f, &lgn)) return false;
   const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
-  const FxXInv kern = fx_xinv_kernel<T>(fx_lgn(f), xi.p && !xi.accumulate && !xi.mean_out && !xi.d2_out);
+  const FxXInv kern = fx_xinv_kernel<T>(lgn, xi.p && !xi.accumulate && !xi.mean_out && !xi.d2_out);
   if (!kern) return false;
   VOFP_LAUNCH(KID_XINV, st, (kern<<<grid, th, sm, st>>>(xi, f)));
   return true;
