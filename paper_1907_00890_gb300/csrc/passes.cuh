@@ -129,15 +129,29 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
-// The same of FP32 partial sums, as FP32 pairs within a warp (32 floats add up exactly in their 48 bits but for the
-// extremes): five shuffled FP64 additions a thread and sum were two FP64 operations a cell.
+// The sum over a warp of FP32 values >= 0, in integers: scaled to the largest exponent they are exact but for bits 2^-58 of
+// the largest value (an FP64 sum drops more), and three 32-bit reductions add them up.  An infinity or a NaN: the FP64 sum.
+__device__ __forceinline__ double warp_sum_exact(float v) {
+  const unsigned b = __float_as_uint(v);
+  const int e = max((int)(b >> 23), 1), emax = __reduce_max_sync(0xffffffffu, e);
+  if (emax >= 255) {  // (also a sign bit, of a NaN)
+    double s = (double)v;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  }
+  const unsigned m = (b & 0x7fffffu) | (b >> 23 ? 0x800000u : 0u);
+  const unsigned long long x = ((unsigned long long)m << 34) >> min(emax - e, 63);
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xfffffu);
+  const unsigned mi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 20) & 0xfffffu);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 40));
+  const long long sum = ((long long)hi << 40) + ((long long)mi << 20) + lo;
+  return (double)sum * __hiloint2double((emax - 150 - 34 + 1023) << 20, 0);
+}
+// The same of FP32 partial sums >= 0: five shuffled FP64 additions a thread and sum were two FP64 operations a cell.
 __device__ __forceinline__ double block_sum(float v, double* red) {
-  ff p(v, 0.0f);
-  for (int o = 16; o > 0; o >>= 1)
-    p += ff(__shfl_down_sync(0xffffffffu, p.hi, o), __shfl_down_sync(0xffffffffu, p.lo, o));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double w = warp_sum_exact(v);
   __syncthreads();
-  if (lane == 0) red[wid] = (double)p;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
   __syncthreads();
   double s = 0;
   if (threadIdx.x == 0) {

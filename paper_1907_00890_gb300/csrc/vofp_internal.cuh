@@ -98,11 +98,12 @@ __device__ __forceinline__ ff neg_if(ff x, bool f) { return ff(neg_if(x.hi, f), 
 __host__ __device__ __forceinline__ bool refine_err_ok(const double* c, int j, double tol2) {
   if (j < 1) return false;  // no estimate from the first solve alone
   const double d0 = c[VOFP_CONV_DEL], dj = c[VOFP_CONV_DEL + j], dp = c[VOFP_CONV_DEL + j - 1];
+  if (!(d0 <= 1.7976931348623157e308)) return false;  // (a norm that has overflowed shows nothing)
   if (dj <= 0.01 * tol2 * d0) return true;
   return dj <= 0.0625 * dp && dj * dj <= 0.01 * tol2 * d0 * dp;
 }
 __host__ __device__ __forceinline__ bool refine_done(const double* c, int k, double tol2) {
-  if (k < 1) return false;
+  if (k < 1 || !(c[0] <= 1.7976931348623157e308)) return false;
   return c[VOFP_CONV_RES + k - 1] <= tol2 * c[0] && refine_err_ok(c, k - 1, tol2);
 }
 // j <= -2: always skipped (a correction beyond an instance's own limit in a batch); j <= 0: never; j >= 1:

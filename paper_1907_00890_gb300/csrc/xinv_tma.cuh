@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kXTmaThreads) k_xinv_tma(const XTmaArgs a, con
     if (threadIdx.x == 0 && s != 0) atomicAdd(x.mean_out, s);
   }
   if (x.d2_out) {
-    const double s = block_sum(acc2f, red);
+    const double s = block_sum((double)acc2f, red);
     if (threadIdx.x == 0 && s != 0) atomicAdd(x.d2_out, s);
   }
 }
