@@ -196,9 +196,9 @@ __device__ __forceinline__ long long fx_of(double x, int E, int rs0, int flip) {
 }
 __device__ __forceinline__ long long fx_of_f32(float x, int E, int rs0, int flip) {
   const int b = __float_as_int(x);
-  const int e = (b >> 23) & 0xff;
-  unsigned long long m = (unsigned long long)(e ? ((unsigned)b << 8) | 0x80000000u : 0u) << 32;
-  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(rs0 + E - (e + 1023 - 127)));
+  const int e = (b >> 23) & 0xff;  // (0: subnormal, 2^-126 as the unit and no implicit bit)
+  unsigned long long m = (unsigned long long)(((unsigned)b << 8) | (e ? 0x80000000u : 0u)) << 32;
+  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(rs0 + E - (max(e, 1) + 1023 - 127)));
   return (b ^ flip) < 0 ? -(long long)m : (long long)m;
 }
 __device__ __forceinline__ long long fx_of(ff x, int E, int rs0, int flip) {
@@ -250,7 +250,8 @@ __device__ __forceinline__ ff fx_to(long long v, int K, int flip, ff*) {
   const int e = 63 - lz + K;  // |value| = u / 2^63 2^e
   if (e < -78 || e > 126) {  // near the ends of the FP32 range
     const double d = fx_to(v, K, flip, (double*)nullptr);
-    return e > 126 ? ff(__int_as_float(0x7f800000 | (s & 0x80000000)), 0.0f) : ff((float)d, (float)(d - (double)(float)d));
+    const float hi = (float)d;
+    return ff(hi, isinf(hi) ? 0.0f : (float)(d - (double)hi));
   }
   const unsigned h = (unsigned)(u >> 32);
   const unsigned hr = ((h >> 8) + ((h >> 7) & 1u));  // 24 bits, or 2^24
