@@ -54,7 +54,7 @@ struct FxDesc {
   int n, nst;
   int bits;   // width of the scaled inputs of a forward pass
   int shift;  // the transform's result is 2^-shift of the exact one
-  int two;    // a rolled odd-prime stage needs a second buffer
+  int two;    // the largest radix of a rolled odd-prime stage, which needs a second buffer and its weights there; 0: none
   int radix[kFxStages];
   // per stage: butterflies per line n / radix, twiddle step n / (Ns radix), and ceil(2^32 / Ns): j / Ns =
   // umulhi(j, magic) for j < 2^16
@@ -83,7 +83,7 @@ inline bool fx_desc(const FftDesc& fd, FxDesc* fx) {
       fx->shift += 2;
     }
     if (R > 5 && R != 8) {
-      fx->two = 1;
+      if (R > fx->two) fx->two = R;
       grow *= 0.25;
       fx->shift += 2;
     }
@@ -141,11 +141,15 @@ __device__ __forceinline__ long long fx_mul(long long a, fxw w, int rd = 1) {
 // (a + i b)(c + i d) / 4 by three products.  Their roundings are centred in the sums (rcpd, rdmc: 0 and 2, less where a
 // factor is 0 or 1 and its product is exact, see fx_twiddle): a constant error of one unit would be added up by the
 // stages that follow into the lowest modes, whose errors the z solve magnifies most.
+// ZERO: a product of zero is zero and needs no centring.  On lines longer than 512, one cell's source (zeros almost
+// everywhere, until the last stage) came out of 2048 points with twice the error of FP64 butterflies in the lowest modes without it.
+template <bool ZERO>
 __device__ __forceinline__ cfx fx_cmul(cfx z, const fxtw& w) {
+  const bool zero = ZERO && (z.x | z.y) == 0;
   const long long k = fx_mul(z.x + z.y, w.c, 0);
   cfx r;
-  r.x = k - fx_mul(z.y, w.cpd, w.rcpd);
-  r.y = k + fx_mul(z.x, w.dmc, w.rdmc);
+  r.x = k - fx_mul(z.y, w.cpd, zero ? 0 : w.rcpd);
+  r.y = k + fx_mul(z.x, w.dmc, zero ? 0 : w.rdmc);
   return r;
 }
 // z / 4, ties to even (also in the place of a product with 1).
@@ -364,7 +368,7 @@ __device__ __noinline__ void fx_stage(int off, int st, int lgB, int NR, int Ns, 
         } else {
 #pragma unroll
           for (int r = 1; r < RAD; ++r) {
-            v[it][r] = fx_cmul(v[it][r], TWS ? tws[r * k * twstep] : twg[r * k * twstep]);
+            v[it][r] = fx_cmul<!TWS>(v[it][r], TWS ? tws[r * k * twstep] : twg[r * k * twstep]);
             fx_fence();
           }
         }
@@ -417,7 +421,7 @@ __device__ __forceinline__ void fx_stage_ct(cfx* buf, const fxtw* __restrict__ t
       } else {
 #pragma unroll
         for (int r = 1; r < RAD; ++r) {
-          v[it][r] = fx_cmul(v[it][r], tw[(r * k) << (LGN - LGNS - lgR)]);
+          v[it][r] = fx_cmul<false>(v[it][r], tw[(r * k) << (LGN - LGNS - lgR)]);
           fx_fence();
         }
       }
@@ -471,13 +475,17 @@ __device__ __forceinline__ long long fx_value(const FxSum& f, int lam) {
 // A rolled stage of an odd prime RAD >= 7 from src into dst (see fft_stage_odd); src is scratch afterwards.  Bound by
 // instruction issue, some 50 a product pair: the weights lie in shared memory with their signs, and the lift of a line
 // with little growth is applied to the sums.
-__device__ __forceinline__ void fx_stage_odd(cfx* src, cfx* dst, int st, int lgB, int n, int Ns, unsigned magic,
-                                             int RAD, const fxtw* __restrict__ tw, int lam) {
-  __shared__ fxq wt[kFxMaxPrime];  // cos, sin of 2 pi a / RAD
+template <bool TWS>
+__device__ __noinline__ void fx_stage_odd(int so, int dof, int st, int lgB, int n, int Ns, unsigned magic, int RAD, int twoff,
+                                          const fxtw* __restrict__ twg, int lam, int wo) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cfx *src = reinterpret_cast<cfx*>(smem_raw + so), *dst = reinterpret_cast<cfx*>(smem_raw + dof);
+  const fxtw* tws = reinterpret_cast<const fxtw*>(smem_raw + twoff);
+  fxq* wt = reinterpret_cast<fxq*>(smem_raw + wo);
   const int NR = n / RAD, H = (RAD - 1) / 2;
   const int mB = (1 << lgB) - 1;
   for (int a = threadIdx.x; a < RAD; a += blockDim.x) {
-    const fxtw w = tw[a * NR];
+    const fxtw w = TWS ? tws[a * NR] : twg[a * NR];
     wt[a] = {w.c, fx_weight(((long long)(w.c.hi - w.cpd.hi) << 32) + ((long long)w.c.lo - w.cpd.lo))};
   }
   if (Ns > 1) {
@@ -489,7 +497,8 @@ __device__ __forceinline__ void fx_stage_odd(cfx* src, cfx* dst, int st, int lgB
       const int j = e - r * NR;
       const int k = j - (int)__umulhi((unsigned)j, magic) * Ns;
       cfx* p = src + e * st + (t & mB);
-      *p = r * k == 0 ? fx_quarter(fx_lift(*p, lam)) : fx_cmul(fx_lift(*p, lam), tw[r * k * twstep]);
+      *p = r * k == 0 ? fx_quarter(fx_lift(*p, lam))
+                      : fx_cmul<!TWS>(fx_lift(*p, lam), TWS ? tws[r * k * twstep] : twg[r * k * twstep]);
     }
   }
   __syncthreads();
@@ -553,7 +562,8 @@ __device__ __forceinline__ cfx* fx_fft_rt(cfx* b0, cfx* b1, int st, int lgB, con
       case 5: fx_stage<5, 2, TWS>(off, st, lgB, fd.nr[s], Ns, fd.step[s], fd.magic[s], to, tw, lam); break;
       case 8: fx_stage<8, 1, TWS>(off, st, lgB, fd.nr[s], Ns, fd.step[s], fd.magic[s], to, tw, lam); break;
       default:
-        fx_stage_odd(off ? b1 : b0, off ? b0 : b1, st, lgB, fd.n, Ns, fd.magic[s], R, tw, lam);
+        fx_stage_odd<TWS>(off, o1 - off, st, lgB, fd.n, Ns, fd.magic[s], R, to, tw, lam,
+                          o1 + fd.n * st * (int)sizeof(cfx) + (TWS ? fd.n * (int)sizeof(fxtw) : 0));
         off = o1 - off;
     }
     Ns *= R;
@@ -644,9 +654,9 @@ __device__ __forceinline__ cfx fx_pre(const cfx* S, int st, int n, int bc, int m
   return cmk<cfx>(Z.x, -Z.y);
 }
 
-// Scaling around the FFT: the inputs are first scaled to `bits` bits; `width` is what the first stage may take (of lines
-// whose sums grow, see fx_settle), `wide` what the step before it hands over; the pre- and post-products leave the
-// result 2^-shift of the exact one.
+// Scaling around the FFT: the inputs are first scaled to `bits` bits (61, or 60 where an inverse pass adds two of them);
+// `width` is what the first stage may take (of lines whose sums grow, see fx_settle), `wide` what the step before it hands
+// over; the pre- and post-products leave the result 2^-shift of the exact one.
 struct FxScale {
   int bits, wide, width, shift;
 };
@@ -655,8 +665,7 @@ __device__ __forceinline__ FxScale fx_scale_of(const FxDesc& fd, int bc, bool in
   const bool quarter = quarter_bc(bc), pre = quarter || (inv && bc != VOFP_BC_P);  // (a product before the FFT)
   // an inverse pass combines two spectra (up to 2 sqrt 2 times larger), or up to sqrt 2 after the product
   s.width = fd.bits - (inv && !quarter ? 1 : 0);
-  s.bits = pre ? 61 : (inv ? 60 : fd.bits);
-  if (s.bits > 61) s.bits = 61;
+  s.bits = inv && !pre ? 60 : 61;
   s.wide = s.bits - (pre ? 2 : 0);
   s.shift = (bc != VOFP_BC_P ? 2 : 0) + (quarter ? 2 : 0);
   return s;
@@ -666,8 +675,11 @@ __device__ __forceinline__ FxScale fx_scale_of(const FxDesc& fd, int bc, bool in
 // are about to be stored: they go in as v >> rho.  The quarter that each product leaves suits lines whose sums grow with
 // every stage.  Where few values dominate -- the spectrum of a smooth line, a right-hand side that is zero but at the
 // interface -- nothing grows past the line's L1 norm, and the quarters would cost accuracy: such a line, with an L1
-// norm of at most 2^5 times its largest value and a larger result that way, goes in with its L1 norm below 2^59 and is
-// lifted again before each product (lam = 2).  `l1`: per line, cleared; units of 2^44.
+// norm of at most 2^5 times its largest value and a larger result that way, goes in with its L1 norm below 2^60 and is
+// lifted again before each product (lam = 2).  (2^60: a lifted value's two parts and their sum stay below 2^63.)  Lines are
+// loaded with all the bits there are and shortened here: loaded at fd.bits, one with a dominating value kept the 5 or 6 bits
+// of headroom it does not need, 4.5e-16 at 512 points and 9e-16 at 2048 where FP64 butterflies err by 2.6e-16 and 3.3e-16; 0.8e-16 and
+// 2.9e-16 this way.  `l1`: per line, cleared; units of 2^44.
 struct FxLine {
   int lam, rho;
 };
@@ -682,7 +694,7 @@ __device__ __forceinline__ FxLine fx_settle(const cfx (&v)[8], int nv, int B, in
   if ((threadIdx.x & 31) < B) atomicAdd(&l1[b], acc);
   __syncthreads();
   const int top = 76 - __clz((int)l1[b]);  // the L1 norm is below 2^top
-  const int over = top > 59 ? top - 59 : 0;
+  const int over = top > 60 ? top - 60 : 0;
   FxLine f;
   if (shift > 0 && top - sc.wide <= 5 && sc.wide - over > sc.width - shift) {
     f.lam = 2;
@@ -720,7 +732,8 @@ __host__ __device__ constexpr int fx_blocks(int lgn) {
   return lgn > 0 ? (896 / fx_ct_threads(lgn) < 1 ? 1 : (896 / fx_ct_threads(lgn) > 24 ? 24 : 896 / fx_ct_threads(lgn))) : 3;
 }
 inline size_t fx_smem(const FxDesc& fd, int lgB, int st) {
-  return (size_t)fd.n * st * sizeof(cfx) * (fd.two ? 2 : 1) + (fd.n <= kFxTwSmem ? (size_t)fd.n * sizeof(fxtw) : 0);
+  return (size_t)fd.n * st * sizeof(cfx) * (fd.two ? 2 : 1) + (fd.n <= kFxTwSmem ? (size_t)fd.n * sizeof(fxtw) : 0) +
+         fd.two * sizeof(fxq);
 }
 
 // ---- passes ----------------------------------------------------------------------------------------------------
