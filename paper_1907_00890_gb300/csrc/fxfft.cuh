@@ -127,33 +127,69 @@ inline double fx_noise(const FftDesc& fd) {
   return sqrt(var) / sig;
 }
 
-// Does a plan (ff: of FP32-pair spectra) transform the length in fd in fixed point?  A rolled stage of a prime p costs p
-// products a value, the floating-point passes' Bluestein form of a prime above 13 two transforms of two to three times
-// the length.  Measured, both, x and y passes, P and NN, in 1e-12 s a value: FP64 at p = 17 (n = 136) 25 against 165-183, 61
-// (122) 50 against 129-148, 151 101 against 150-158, 197 135 against 186-198, 251 172 against 133-162; FP32 pairs at p = 17
-// 26 against 57, 47 (188) 44 against 50, 53 (106) 48 against 62, 61 (122) 52 against 44 (its convolution has a lucky 256
-// points), 79 (158) 66 against 50.
-// Other lengths on small grids: a pass is one short wave of blocks, bound by the latency of its chain, and that of the
-// fixed-point passes is the longer one.  Measured, one pass, floating point against fixed point: FP64, lengths without a
-// compiled-in kernel, x 48 (110592 cells) 1 : 0.81-1.00, 24 (144000) 0.80-0.95, 96 (221088) 1.11-1.15, y 20 (64000) 0.8, 48
-// (110592) 0.8, 24 (198144) 0.90, 96 (209664) 1.24, but 384 (98304) 2.0; compiled-in 64 (65536) 1.05-1.3; 32, a warp per block: a
-// 32^3 projection 64 -> 53 us, x 61440 cells 0.90-1.02, 173376 0.74-0.96, y 86016 0.91, 326656 1.26.  FP32 pairs, any length: x 48
-// (110592) 0.66-0.73, 64 (336896) 0.83-1.20, 72 (460800) 0.90-1.05, y 96 (61440) 0.7, 192 (380160) 0.96; without a compiled-in
-// kernel, x 80 (512000) 0.78-0.91, 100 (864000) 0.81-0.96, y 96 (864000) 0.73-0.78; 32 x 128 x 128 no slower.
+// Lines of a compiled-in length's tile (2^lgn samples).
+__host__ __device__ constexpr int fx_ct_lgB(int lgn) { return lgn == 5 ? 1 : 3; }
+// Tile width, from the number of eight-line tiles: the widest of 8, 4, 2, 1 lines whose tile takes at most 256
+// threads (512 for 512 samples),
+// narrowed while tiles are fewer than SMs (but not below `least` lines, nor a warp with two values a lane).
+inline int fx_lgB(int n, long tiles8, int least) {
+  int lg = 3;
+  while (lg > 0 && (n << lg) > ((n & (n - 1)) == 0 && n <= 512 ? 4096 : 2048)) --lg;
+  while (lg > least && (tiles8 << (3 - lg)) < 152 && (n << lg) > 64) --lg;
+  return lg;
+}
+// Eight-line tiles of the x, or the y pass.
+inline long fx_tiles8(int nx, int ny, int nz, bool y) {
+  return y ? (long)((nx + 15) / 16) * nz : (((long)ny * nz + 1) / 2 + 7) / 8;
+}
+
+// Does a plan (ff: of FP32-pair spectra) transform the x (or y) axis of the length in fd in fixed point?  Where it is the
+// faster way, by cells.  Measured per axis, forward and inverse pass together, P and NN, floating point against fixed point (above 1:
+// fixed point is faster).
+// Powers of two.  FP64 from 64 on: 0.94-1.5 below 400,000 cells, 1.4-3.8 above; 32: 1.2-1.4 where the compiled-in kernel's one-warp
+// tiles are what the grid has (16,000 and 32,000 cells), 0.79-0.97 from 64,000 to 256,000 with the run-time kernel, 1.1-2.0 from 512,000.
+// FP32 pairs, x (their y pass takes TMA tiles): 64 0.87-1.06 below 480,000, 1.06-1.7 above; 128, 256, 512 0.73-0.99 up to 600,000,
+// 1.0-1.15 at 720,000, 1.2-1.5 above a million.
+// Other lengths.  A pass of a small grid is one short wave of blocks, bound by the latency of its chain, and that of the
+// fixed-point passes is the longer one.  FP64: 0.70-0.99 at 128,000 cells on lines below 64, 1.0-1.4 at 200,000 to 250,000 -- but for
+// three short stages (30: 0.74-0.87, 48: 0.9, 60: 0.84-1.0; 0.94-1.3 at 300,000) -- and 1.3-2.6 above 500,000; y of 256 and more
+// 1.4-2.2 everywhere.  FP32 pairs, x: 0.6-0.95 up to 500,000 cells, 0.81-1.2 at 2,000,000, 0.87-1.16 at 2,400,000, 1.0-1.28 at
+// 2,800,000, 1.1-1.4 at 12,000,000; y: up to 50 samples 1.0-1.28 from 2,400,000, 72 to 100 0.74-1.08 below 6,000,000 and 1.0-1.2 at 8 to 12
+// million, beyond that 0.66-0.98 up to 6,000,000 and 0.87-1.1 at 8 to 12.
+// Lengths with a prime above 13: a rolled stage costs p products a value, the floating-point passes' Bluestein form two
+// transforms of two to three times the length.  FP64: p up to 89 0.9-2.3 below 250,000 cells, 1.3-4.9 above; 97 to 113 on x 0.78-1.35 below
+// 250,000, 1.2-2.6 above; 127 to 199 0.54-1.0 below 500,000, 1.03-2.4 above; y 1.0-6.6.  FP32 pairs: p up to 43 0.86-2.4; 47 and
+// 53 0.76-1.1 from 64,000 to 250,000, 0.92-1.5 above.  Where a one-warp block holds at most 128 values, four a lane, the chain
+// is short enough for any of them: 1.0-1.9.
 // `force` (VOFP_FX=1 when the plan is created): fixed point whatever the grid, for comparisons.
-inline bool fx_takes(const FftDesc& fd, bool ff, bool y, long cells, bool force) {
+inline bool fx_takes(const FftDesc& fd, bool ff, bool y, int nx, int ny, int nz, bool force) {
   FxDesc fx;
-  for (int s = 0; s < fd.nst; ++s)
+  int prime = 1;
+  for (int s = 0; s < fd.nst; ++s) {
     if (fd.radix[s] > (ff ? 53 : kFxMaxPrime)) return false;
+    if (fd.radix[s] != 8 && fd.radix[s] != 4 && fd.radix[s] > prime) prime = fd.radix[s];
+  }
   if (!fx_desc(fd, &fx)) return false;
   // (stages of radix 3 err more in FP64 too; a Bluestein form by 4e-16 to 7e-16)
   if (!fd.bm && !ff && fx_noise(fd) > (fx.two ? 1.45e-16 : 2e-16)) return false;
-  if (force || fd.bm) return true;
-  const bool pow2 = (fd.n & (fd.n - 1)) == 0;
-  if (ff) return cells >= (pow2 && fd.n >= 32 && fd.n <= 512 ? 480000 : 2000000);
-  if (pow2 && fd.n >= 64 && fd.n <= 512) return true;
-  if (fd.n == 32) return cells <= 48000 || cells >= (y ? 200000 : 480000);
-  return cells >= 200000 || (y && fd.n >= 256);
+  if (force) return true;
+  const long cells = (long)nx * ny * nz;
+  const int n = fd.n, lgB = fx_lgB(n, fx_tiles8(nx, ny, nz, y), y ? 1 : 0);
+  if (fd.bm) {
+    if ((n << lgB) <= 128) return true;
+    if (ff) return prime <= 43 || cells >= 500000;
+    return y || prime <= 89 || cells >= (prime <= 113 ? 250000 : 500000);
+  }
+  const bool pow2 = (n & (n - 1)) == 0;
+  if (pow2 && n >= 32 && n <= 512) {
+    if (ff) return cells >= (n <= 64 ? 480000 : 700000);
+    return n >= 64 || lgB == fx_ct_lgB(5) || cells >= 480000;
+  }
+  if (ff) {
+    if (y) return cells >= 2400000 && (n <= 50 || (n <= 100 && cells >= 8000000));
+    return cells >= 2800000;
+  }
+  return cells >= (n < 64 && fd.nst >= 3 ? 300000 : 200000) || (y && n >= 256);
 }
 
 // ---- scalars ------------------------------------------------------------------------------------------------
@@ -422,7 +458,6 @@ __device__ __noinline__ void fx_stage(int off, int st, int lgB, int NR, int Ns, 
 }
 
 // The same for a power-of-two length 2^LGN, its tile width and threads known at compile time.
-__host__ __device__ constexpr int fx_ct_lgB(int lgn) { return lgn == 5 ? 1 : 3; }
 __host__ __device__ constexpr int fx_ct_threads(int lgn) {
   return (1 << (lgn + fx_ct_lgB(lgn))) / 8 < 32 ? 32 : (1 << (lgn + fx_ct_lgB(lgn))) / 8;
 }
@@ -738,16 +773,6 @@ __device__ __forceinline__ FxLine fx_settle(const cfx (&v)[8], int nv, int B, in
 __device__ __forceinline__ cfx fx_down(cfx v, int rho) {
   const long long h = (1ll << rho) >> 1;
   return cmk<cfx>((v.x + h) >> rho, (v.y + h) >> rho);
-}
-
-// Tile width, from the number of eight-line tiles: the widest of 8, 4, 2, 1 lines whose tile takes at most 256
-// threads (512 for 512 samples),
-// narrowed while tiles are fewer than SMs (but not below `least` lines, nor a warp with two values a lane).
-inline int fx_lgB(int n, long tiles8, int least) {
-  int lg = 3;
-  while (lg > 0 && (n << lg) > ((n & (n - 1)) == 0 && n <= 512 ? 4096 : 2048)) --lg;
-  while (lg > least && (tiles8 << (3 - lg)) < 152 && (n << lg) > 64) --lg;
-  return lg;
 }
 
 // Threads for a tile of 2^lgB lines of n: an eighth of its values, whole warps.

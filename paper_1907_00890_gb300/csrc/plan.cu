@@ -302,7 +302,7 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     p->ax[a].n = n;
     p->ax[a].bc = bc[a];
     if (p->ax[a].fd.bm) blu[a] = bluestein_tables(p->ax[a].fd);
-    if (o.prec != VOFP_MIXED && fx_takes(p->ax[a].fd, o.prec == VOFP_FF, a == 1, (long)nx * ny * nz, fx_force)) {
+    if (o.prec != VOFP_MIXED && fx_takes(p->ax[a].fd, o.prec == VOFP_FF, a == 1, nx, ny, nz, fx_force)) {
       twfx[a].resize(n);
       quartfx[a].resize(nq);
       for (int q = 0; q < n; ++q) {
