@@ -65,11 +65,16 @@ constexpr size_t kYTmaTile = std::is_same<R, double>::value ? (size_t)112 * 1024
 // active); two CTAs took the FP32 inverse passes of a 512^3 solve from 2.73 to 2.30 ms.  NULL for other
 // lengths.
 typedef void (*XTmaKernel)(const XTmaArgs, const CUtensorMap, const CUtensorMap);
-static int xtma_lgB(int lgn) { return lgn >= 9 ? 2 : 3; }
+template <typename R>
+static int xtma_lgB(int lgn) {
+  return std::is_same<R, float>::value ? (lgn >= 9 ? 2 : 3) : (lgn >= 9 ? 2 : (lgn == 8 ? 3 : 4));
+}
+template <typename R>
 static XTmaKernel xtma_kernel(int lgn) {
-  if (lgn == 9) return k_xinv_tma<float, 9, 2>;
-  if (lgn == 8) return k_xinv_tma<float, 8, 3>;
-  if (lgn == 7) return k_xinv_tma<float, 7, 3>;
+  constexpr bool F = std::is_same<R, float>::value;
+  if (lgn == 9) return k_xinv_tma<R, 9, 2>;
+  if (lgn == 8) return k_xinv_tma<R, 8, 3>;
+  if (lgn == 7) return F ? k_xinv_tma<R, 7, 3> : k_xinv_tma<R, 7, 4>;
   return nullptr;
 }
 
@@ -99,7 +104,8 @@ void init_kernel_attributes_mixed() {
                              kYTmaSmem);
       }
   for (int lgn = 7; lgn <= 9; ++lgn) {
-    cudaFuncSetAttribute(xtma_kernel(lgn), cudaFuncAttributeMaxDynamicSharedMemorySize, kYTmaSmem);
+    cudaFuncSetAttribute(xtma_kernel<float>(lgn), cudaFuncAttributeMaxDynamicSharedMemorySize, kYTmaSmem);
+    cudaFuncSetAttribute(xtma_kernel<ff>(lgn), cudaFuncAttributeMaxDynamicSharedMemorySize, kYTmaSmem);
   }
 }
 
@@ -171,31 +177,32 @@ static void ytma_setup(vofp_plan* pl, void* spectrum) {
 
 // First use of the TMA inverse x pass: nx of 128, 256 or 512 (VOFP_X_TMA=0 switches it off); the tensor map
 // views the spectrum as {min(nx, 256), nx / min(nx, 256), ny nz} so that one box is a tile of whole lines.
+template <typename R>
 static void xtma_setup(vofp_plan* pl) {
   pl->xtma_state = -1;
   const char* env = getenv("VOFP_X_TMA");
   if (env && env[0] == '0') return;
   const int nx = pl->n[0];
   if (nx != 128 && nx != 256 && nx != 512) return;
-  const int lgn = 31 - __builtin_clz((unsigned)nx), lgB = xtma_lgB(lgn);
+  const int lgn = 31 - __builtin_clz((unsigned)nx), lgB = xtma_lgB<R>(lgn);
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return;
   const int h = nx < 256 ? nx : 256;
   const long nlines = (long)pl->n[1] * pl->n[2];
   CUtensorMap tm;
   const cuuint64_t dims[3] = {(cuuint64_t)h, (cuuint64_t)(nx / h), (cuuint64_t)nlines};
-  const cuuint64_t strides[2] = {(cuuint64_t)h * sizeof(float), (cuuint64_t)nx * sizeof(float)};
+  const cuuint64_t strides[2] = {(cuuint64_t)h * sizeof(R), (cuuint64_t)nx * sizeof(R)};
   const cuuint32_t box[3] = {(cuuint32_t)h, (cuuint32_t)(nx / h), (cuuint32_t)(2 << lgB)};
   const cuuint32_t estr[3] = {1, 1, 1};
-  if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, pl->S32, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-      CUDA_SUCCESS)
+  const CUtensorMapDataType dt = sizeof(R) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
+  if (enc(&tm, dt, 3, pl->S32, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return;
   int per_sm = 0, nsm = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xtma_kernel(lgn), kXTmaThreads,
-                                                    xtma_smem_bytes(nx, lgB, sizeof(float), true)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xtma_kernel<R>(lgn), kXTmaThreads,
+                                                    xtma_smem_bytes(nx, lgB, sizeof(R), true)) != cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     return;
@@ -223,15 +230,16 @@ static bool xtma_potential_map(int nx, long nlines, double* p, int lgB, CUtensor
          CUDA_SUCCESS;
 }
 
+template <typename R>
 static bool xinv_tma(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
-  if (pl->xtma_state == 0) xtma_setup(pl);
+  if (pl->xtma_state == 0) xtma_setup<R>(pl);
   if (pl->xtma_state != 1) return false;
   CUtensorMap tm, tp;
   memcpy(&tm, pl->xtma_map, sizeof(tm));
   const int lgn = 31 - __builtin_clz((unsigned)pl->n[0]);
   XTmaArgs ta;
   ta.xi = xi;
-  ta.lgB = xtma_lgB(lgn);
+  ta.lgB = xtma_lgB<R>(lgn);
   ta.info = pl->info;
   const bool acc = xi.p && xi.accumulate;
   if (acc) {
@@ -239,8 +247,8 @@ static bool xinv_tma(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
   } else {
     tp = tm;  // not read
   }
-  const size_t sm = xtma_smem_bytes(pl->n[0], ta.lgB, sizeof(float), acc);
-  VOFP_LAUNCH(KID_XINV, st, (xtma_kernel(lgn)<<<pl->xtma_grid, kXTmaThreads, sm, st>>>(ta, tm, tp)));
+  const size_t sm = xtma_smem_bytes(pl->n[0], ta.lgB, sizeof(R), acc);
+  VOFP_LAUNCH(KID_XINV, st, (xtma_kernel<R>(lgn)<<<pl->xtma_grid, kXTmaThreads, sm, st>>>(ta, tm, tp)));
   return true;
 }
 
@@ -415,9 +423,9 @@ static void xinv_red(vofp_plan* pl, double* pout, int accumulate, int skip_k, do
   if (std::is_same<R, float>::value && xtc_xinv(pl, xi, st)) return;  // tensor-core transform
   if constexpr (std::is_same<R, ff>::value) {
     if (fx_xinv<ff>(pl, xi, st)) return;  // fixed point
-  } else if (xinv_tma(pl, xi, st)) {  // TMA-staged tiles
-    return;
   }
+  // TMA-staged tiles (FP32 pairs: grids that fx_takes leaves out; 256 x 32 x 32 13.4 us, 22.6 on gathered tiles)
+  if (xinv_tma<R>(pl, xi, st)) return;
   const int xgrid = xpass_blocks(xi.ny, xi.nz, xi.pb);
   const size_t xsm = 2 * (size_t)xi.pb * fft_span(xi.fd, xi.blu) * sizeof(C);
   VOFP_LAUNCH(KID_XINV, st, (xinv_kernel<R, C>()<<<xgrid, 256, xsm, st>>>(xi)));
