@@ -20,10 +20,7 @@ static int fx_lgn(const FxTables& f) {
   // (FP32-pair plans leave the grids of one-warp tiles of 32 samples to the floating-point passes, see fx_takes)
   if ((n & (n - 1)) || n < (std::is_same<T, double>::value ? 32 : 64) || n > 512) return 0;
   const int lgn = 31 - __builtin_clz((unsigned)n);
-  if (f.lgB != fx_ct_lgB(lgn)) return 0;
-  for (int s = 0; s < f.fd.nst; ++s)  // (an autotuned stage order keeps the run-time kernel)
-    if (f.fd.radix[s] != fx_radix(lgn, s)) return 0;
-  return lgn;
+  return f.lgB == fx_ct_lgB(lgn) ? lgn : 0;  // (the stages are the plan's: see fx_radix)
 }
 typedef void (*FxXFwd)(const XArgs, const FxTables);
 typedef void (*FxYPass)(const YArgs, const FxTables);

@@ -4,9 +4,10 @@
 // walking each knob in turn -- line pairs per block of the x passes, columns per block of the y passes, the
 // z kernel (segmented tiles, shared-memory staged chains, or streamed chains with their systems per block),
 // and the order of the FFT radix stages on x and on y (the plan's factorisation or its reverse) -- and keeps
-// the fastest value of each (coordinate descent over the candidates that fit in shared memory).  Results are cached per process and, when the environment
-// variable VOFP_TUNE_CACHE names a file, in that file (one line per grid/precision/GPU key), so a serving
-// process or a batch pays the search once per shape.
+// the fastest value of each (coordinate descent over the candidates that fit in shared memory).  An axis that is transformed
+// in fixed point has its tile and stage order from its length and the grid: its knobs are left alone, as is the z knob of
+// circulant systems.  Results are cached per process and, when the environment variable VOFP_TUNE_CACHE names a file, in that
+// file (one line per grid/precision/GPU key), so a serving process or a batch pays the search once per shape.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -66,6 +67,9 @@ void save_entry(const std::string& k, const Shape& s) {
 // the reduced-precision (refinement) paths keep their shapes in ytx32 / zti32
 bool mixed(const vofp_plan* p) { return p->opts.prec != VOFP_FP64; }
 
+// The axes (bit 0: x, bit 1: y) in fixed point.
+int fx_axes(const vofp_plan* p) { return (p->ax[0].twfx ? 1 : 0) | (p->ax[1].twfx ? 2 : 0); }
+
 // Reverse the radix sequence of an axis (any order of the stages gives the same transform, up to rounding).
 void reverse_stages(vofp::FftDesc& fd) {
   for (int a = 0, b = fd.nst - 1; a < b; ++a, --b) {
@@ -75,7 +79,8 @@ void reverse_stages(vofp::FftDesc& fd) {
   }
 }
 
-void apply(vofp_plan* p, const Shape& s) {
+void apply(vofp_plan* p, Shape s) {
+  s.ord &= ~fx_axes(p);  // (an entry made before those axes ran in fixed point)
   for (int a = 0; a < 2; ++a)
     if (((s.ord ^ p->radix_order) >> a) & 1) reverse_stages(p->ax[a].fd);
   p->radix_order = s.ord;
@@ -113,22 +118,40 @@ bool fits(const vofp_plan* p, const Shape& s) {
   return (size_t)3 * s.zti * p->n[2] * r <= lim;
 }
 
-// Average milliseconds of a Poisson solve of the plan's scratch potential (in place).
+// A bounded, deterministic right-hand side: noise in [-1, 1) (a transform of zeros takes no arithmetic).
+__global__ void k_fill(double* p, size_t n) {
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
+    unsigned h = (unsigned)t * 2654435761u;
+    h = (h ^ (h >> 15)) * 2246822519u;
+    p[t] = (int)(h ^ (h >> 13)) * 0x1p-31;
+  }
+}
+
+// Average milliseconds of a Poisson solve of the plan's scratch potential (in place, filled before each).
 float time_solve(vofp_plan* p, cudaStream_t st) {
-  cudaEvent_t a, b;
-  cudaEventCreate(&a);
-  cudaEventCreate(&b);
   const int reps = 4;
-  vofp_poisson_solve(p, p->P, p->P, st, nullptr);
-  cudaEventRecord(a, st);
-  for (int r = 0; r < reps; ++r) vofp_poisson_solve(p, p->P, p->P, st, nullptr);
-  cudaEventRecord(b, st);
-  cudaEventSynchronize(b);
-  float ms = 0;
-  cudaEventElapsedTime(&ms, a, b);
-  cudaEventDestroy(a);
-  cudaEventDestroy(b);
-  return ms / reps;
+  const size_t cells = (size_t)p->n[0] * p->n[1] * p->n[2];
+  cudaEvent_t a[reps], b[reps];
+  for (int r = 0; r < reps; ++r) {
+    cudaEventCreate(&a[r]);
+    cudaEventCreate(&b[r]);
+  }
+  for (int r = -1; r < reps; ++r) {  // (one to warm up)
+    k_fill<<<vofp::grid_blocks(cells, 256), 256, 0, st>>>(p->P, cells);
+    if (r >= 0) cudaEventRecord(a[r], st);
+    vofp_poisson_solve(p, p->P, p->P, st, nullptr);
+    if (r >= 0) cudaEventRecord(b[r], st);
+  }
+  float sum = 0;
+  for (int r = 0; r < reps; ++r) {
+    float ms = 0;
+    cudaEventSynchronize(b[r]);
+    cudaEventElapsedTime(&ms, a[r], b[r]);
+    sum += ms;
+    cudaEventDestroy(a[r]);
+    cudaEventDestroy(b[r]);
+  }
+  return sum / reps;
 }
 
 }  // namespace
@@ -147,15 +170,15 @@ extern "C" int vofp_plan_tune(vofp_plan* p) {
   }
   cudaStream_t st;
   if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return VOFP_ERR_CUDA;
-  // a bounded, deterministic right-hand side: zeros (the kernels' cost does not depend on the values)
-  cudaMemsetAsync(p->P, 0, sizeof(double) * (size_t)p->n[0] * p->n[1] * p->n[2], st);
   Shape best = current(p);
   float tbest = time_solve(p, st);
   const int xs[] = {1, 2, 4, 8, 16, 32};
   const int ys[] = {2, 4, 8, 16, 32};
   const int zs[] = {-1, -2, 0, 8, 16, 32, 64, 128};
   const int os[] = {0, 1, 2, 3};
+  const int fx = fx_axes(p);
   for (int knob = 0; knob < 4; ++knob) {
+    if ((knob == 0 && (fx & 1)) || (knob == 1 && (fx & 2)) || (knob == 2 && p->zcirc)) continue;
     const int* cand = knob == 0 ? xs : (knob == 1 ? ys : (knob == 2 ? zs : os));
     const int nc = knob == 0 ? 6 : (knob == 1 ? 5 : (knob == 2 ? 8 : 4));
     for (int c = 0; c < nc; ++c) {
@@ -164,7 +187,7 @@ extern "C" int vofp_plan_tune(vofp_plan* p) {
       if (knob == 1) s.ytx = cand[c];
       if (knob == 2) s.zti = cand[c];
       if (knob == 3) s.ord = cand[c];
-      if (!fits(p, s)) continue;
+      if (!fits(p, s) || (s.ord & fx)) continue;
       apply(p, s);
       const float t = time_solve(p, st);
       if (t < tbest) {
