@@ -591,7 +591,7 @@ int plan_prepare(int nx, int ny, int nz, double dx, double dy, const double* dz,
     // or 128 threads' columns fit in 96 KB, else kept in place in the spectrum)
     auto table_ti = [&](size_t elem, bool fp64) {
       if (!fp64 && ztab_seg_code(nz, elem) != 0) return ztab_seg_code(nz, elem);
-      if (ztab_use_staged(nx, ny, nz, elem)) return 0;
+      if (ztab_use_staged(nx, ny, nz, elem, fp64, p->singular)) return 0;
       if ((size_t)128 * nz * elem <= 96 * 1024) return 128;
       if ((size_t)64 * nz * elem <= 96 * 1024) return 64;
       return 128;

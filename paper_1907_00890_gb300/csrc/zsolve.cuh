@@ -714,9 +714,17 @@ static __global__ void __launch_bounds__(128) k_zlow_scan(ZArgs a, const int2* _
 constexpr int kZStagedTI = 32;
 inline size_t ztab_staged_smem(int nz, size_t elem) { return (size_t)nz * (kZStagedTI + 1) * elem; }
 // Staged kernel for FP64 / FP32-pair arithmetic when the grid has fewer than 152 * 256 systems (too few to
-// hide the recurrences' latency one thread each) and the tile fits in shared memory.
-inline bool ztab_use_staged(int nx, int ny, int nz, size_t elem) {
-  return (size_t)nx * ny < (size_t)152 * 256 && ztab_staged_smem(nz, elem) <= 200 * 1024;
+// hide the recurrences' latency one thread each) and the tile fits in shared memory.  Above 438 rows an SM holds one tile:
+// its chains overlap no others and its load and store no chain, and the streaming kernel is the faster one from five tiles an
+// SM on (FP32 pairs: seven), unless it has the mean mode of an FP64 plan, which it solves serially.  Measured, staged against
+// streaming, us: FP64 DD, NN, DD 190 x 200 x 400 408 / 466, x 440 657 / 515, x 600 989 / 702, 800 tiles of 700 rows 840 / 800, 640 645 /
+// 762; P, P, NN 190 x 200 x 440 572 / 924; FP32 pairs DD, NN, DD x 440 543 / 516, 1000 tiles of 700 rows 796 / 803, 800 665 / 805.
+inline bool ztab_use_staged(int nx, int ny, int nz, size_t elem, bool fp64, bool singular) {
+  const size_t sm = ztab_staged_smem(nz, elem);
+  if ((size_t)nx * ny >= (size_t)152 * 256 || sm > 200 * 1024) return false;
+  const long tiles = (long)((nx + kZStagedTI - 1) / kZStagedTI) * ny;
+  if (sm <= 113 * 1024 || (fp64 && singular)) return true;
+  return tiles <= 152 * (fp64 ? 5 : 7);
 }
 
 // Both recurrences of one column yc (stride TI) of the tile; F: its factors at stride ts.
