@@ -15,24 +15,47 @@ __host__ __device__ __forceinline__ size_t total_faces(const GridDev& g) {
          (size_t)g.nx * g.ny * nface(g.nz, g.bcz);
 }
 
-// ---- the faces at the low corners of a tile of cells ------------------------------------------------------------------
-// The face kernels take a tile of 32 x kCornerRows corners of one plane, a warp per row: at corner (i, j, k) the x, y and z
-// face there (the last face of a bounded axis belongs to a corner past the last cell).  The cell fields the three share
-// come from L1 after the first, and offsets are 32-bit (a plan has fewer than 2^31 cells).
+// ---- the faces at the low corners of cells --------------------------------------------------------------------------
+// A thread of a face kernel takes the x, y and z face at the corner (i, j, k) of cells (the last face of a bounded axis belongs
+// to a corner past the last cell).  The cell fields the three share come from L1 after the first, and offsets are 32-bit (a
+// plan has fewer than 2^31 cells).  Lanes run over the corners of a plane, row after row; while the blocks are fewer than
+// eight an SM, a block takes the faces of one axis, so that a thread's chain is one face's loads and not three.
+// (Tiles of 32 x 16 corners, a warp per row, leave lanes idle where a row is no multiple of 32 and make a warp wait for each
+// row in turn: extension of 128^3 51.8 us on tiles, 39.1 flat; 20 x 20 x 160 12.0, 9.2; 33 x 33 x 300 30.0, 18.2; variable-density
+// pass of 128^3 86, 74.)
+constexpr int kCornerThreads = 128;
+inline dim3 flat_grid(const GridDev& g) {
+  const unsigned bx = (unsigned)((nface(g.nx, g.bcx) * nface(g.ny, g.bcy) + kCornerThreads - 1) / kCornerThreads);
+  const unsigned nz = (unsigned)nface(g.nz, g.bcz);
+  return dim3(bx, 1, (long)bx * nz < 1216 ? 3 * nz : nz);
+}
+// This thread's corner and plane (returned), and the axes it takes (a bit each).
+__device__ __forceinline__ int flat_corner(const GridDev& g, int& i, int& j, int& axes) {
+  const int nz = nface(g.nz, g.bcz), c = blockIdx.x * kCornerThreads + threadIdx.x, fx = nface(g.nx, g.bcx);
+  j = c / fx;
+  i = c - j * fx;
+  axes = 7;
+  if (gridDim.z == nz) return blockIdx.z;
+  const int a = blockIdx.z / nz;
+  axes = 1 << a;
+  return blockIdx.z - a * nz;
+}
+
+// The velocity correction's other layout: a tile of 32 x kCornerRows corners of one plane, a warp per row, where its rows fill the
+// warps; it moves the most bytes an operation, and a warp on one row moves them in fewer sectors (256 x 256 x 128 104 us on
+// tiles, 116 flat; 250 x 150 x 128 65.4, 69.2).  Flat: tiles fewer than four an SM (20 x 20 x 160 8.7, 6.8) or a tenth of their
+// lanes idle (130 x 130 x 128 41.0, 34.4; 33 x 33 x 300 16.1, 11.3; 200 x 200 x 60, 14% idle, 40.8, 38.4).
 constexpr int kCornerRows = 16;
 __host__ __device__ __forceinline__ int corner_tiles_x(const GridDev& g) { return (nface(g.nx, g.bcx) + 31) >> 5; }
 __host__ __device__ __forceinline__ int corner_tiles_y(const GridDev& g) {
   return (nface(g.ny, g.bcy) + kCornerRows - 1) / kCornerRows;
 }
-constexpr int kCornerThreads = 512;  // at most
-// Threads per tile: four warps of four rows each; sixteen of one row while the tiles are fewer than four per SM, all of them
-// resident (a 32^3 correction took 5 us longer with four; the extension of 20 x 20 x 160, 320 tiles: 16.6 us with four, 12.4 with
-// sixteen).
-inline int corner_threads(const GridDev& g) {
-  return (long)corner_tiles_x(g) * corner_tiles_y(g) * nface(g.nz, g.bcz) < 608 ? 512 : 128;
-}
 inline dim3 corner_grid(const GridDev& g) {
   return dim3((unsigned)corner_tiles_x(g), (unsigned)corner_tiles_y(g), (unsigned)nface(g.nz, g.bcz));
+}
+inline bool corner_flat(const GridDev& g) {
+  const long tiles = (long)corner_tiles_x(g) * corner_tiles_y(g);
+  return tiles * nface(g.nz, g.bcz) < 608 || 10L * nface(g.nx, g.bcx) * nface(g.ny, g.bcy) < 9 * tiles * 32 * kCornerRows;
 }
 
 // Double a normal value by its exponent.
@@ -95,13 +118,16 @@ __device__ __forceinline__ void grad_face(const GridDev& g, const double* __rest
   if (AXIS != 2 && r.e > 0) c = twice(c);
   F[r.off] = fma(-c, face_diff(p, r), F[r.off]);
 }
-__device__ __forceinline__ void grad_tile(const GridDev& g, const double* __restrict__ p, double* u, double* v, double* w,
-                                          double s, double sx, double sy, int tx, int ty, int k) {
-  const int i = tx * 32 + (threadIdx.x & 31);
+__device__ __forceinline__ double grad_sz(const GridDev& g, double s, int k) {
   // (half the end cell's width at a D end)
   const bool dlo = k == 0 && (g.bcz == VOFP_BC_DD || g.bcz == VOFP_BC_DN);
   const bool dhi = k == g.nz && (g.bcz == VOFP_BC_DD || g.bcz == VOFP_BC_ND);
-  const double sz = s * face_rdist<2>(g, k, dlo ? 1 : (dhi ? 2 : 0));
+  return s * face_rdist<2>(g, k, dlo ? 1 : (dhi ? 2 : 0));
+}
+__device__ __forceinline__ void grad_tile(const GridDev& g, const double* __restrict__ p, double* u, double* v, double* w,
+                                          double s, double sx, double sy, int tx, int ty, int k) {
+  const int i = tx * 32 + (threadIdx.x & 31);
+  const double sz = grad_sz(g, s, k);
   for (int q = threadIdx.x >> 5; q < kCornerRows; q += blockDim.x >> 5) {
     const int j = ty * kCornerRows + q;
     grad_face<0>(g, p, u, sx, i, j, k);
@@ -109,10 +135,19 @@ __device__ __forceinline__ void grad_tile(const GridDev& g, const double* __rest
     grad_face<2>(g, p, w, sz, i, j, k);
   }
 }
+template <bool FLAT>
 static __global__ void __launch_bounds__(kCornerThreads) k_grad_update(GridDev g, const double* __restrict__ p, double* u,
                                                                        double* v, double* w, double s, double sx,
                                                                        double sy) {
-  grad_tile(g, p, u, v, w, s, sx, sy, blockIdx.x, blockIdx.y, blockIdx.z);
+  if (FLAT) {
+    int i, j, axes;
+    const int k = flat_corner(g, i, j, axes);
+    if (axes & 1) grad_face<0>(g, p, u, sx, i, j, k);
+    if (axes & 2) grad_face<1>(g, p, v, sy, i, j, k);
+    if (axes & 4) grad_face<2>(g, p, w, grad_sz(g, s, k), i, j, k);
+  } else {
+    grad_tile(g, p, u, v, w, s, sx, sy, blockIdx.x, blockIdx.y, blockIdx.z);
+  }
 }
 
 // Interface geometry per cell: s = coef * mdot * |grad C| and n = -grad C / |grad C| (clipped).  Away from the interface
@@ -142,10 +177,13 @@ __device__ __forceinline__ void store_normal(const GridDev& g, bool act, unsigne
   }
 }
 
-// Launch shape: a warp per row of 32 cells, four rows a block, marching kGeoPlanes planes (C of three planes in registers).
+// Launch shape: a warp per row of 32 cells, four rows a block, marching kGeoPlanes planes (C of three planes in registers); one
+// plane while the blocks are fewer than four an SM, each plane's loads waiting for the last one's.
 constexpr int kGeoPlanes = 4;
 inline dim3 geometry_grid(const GridDev& g) {
-  return dim3((unsigned)mask_words(g.nx), (unsigned)((g.ny + 3) / 4), (unsigned)((g.nz + kGeoPlanes - 1) / kGeoPlanes));
+  const unsigned bx = (unsigned)mask_words(g.nx), by = (unsigned)((g.ny + 3) / 4);
+  const unsigned bz = (unsigned)((g.nz + kGeoPlanes - 1) / kGeoPlanes);
+  return dim3(bx, by, (long)bx * by * bz < 608 ? (unsigned)g.nz : bz);
 }
 // FF: everything after the C differences in FP32 pairs (reduced-precision plans, central differences) -- scaling,
 // |grad C|^2, the reciprocal square root (FP32 seed and one FP32-pair Newton step), s and n -- with integer-pipe
@@ -157,7 +195,8 @@ static __global__ void __launch_bounds__(128) k_geometry(GridDev g, const double
                                                         double* __restrict__ ny, double* __restrict__ nz,
                                                         unsigned* __restrict__ mask) {
   const int i = blockIdx.x * 32 + (threadIdx.x & 31), j = blockIdx.y * 4 + (threadIdx.x >> 5);
-  const int k0 = blockIdx.z * kGeoPlanes, k1 = k0 + kGeoPlanes < g.nz ? k0 + kGeoPlanes : g.nz;
+  const int planes = gridDim.z == g.nz ? 1 : kGeoPlanes;
+  const int k0 = blockIdx.z * planes, k1 = k0 + planes < g.nz ? k0 + planes : g.nz;
   const bool act = i < g.nx && j < g.ny;
   const unsigned plane = (unsigned)g.nx * g.ny;
   // in-plane offsets of the neighbours (clamped at bounded ends, wrapped at periodic ones), x fastest
@@ -282,16 +321,14 @@ __device__ __forceinline__ void extend_face(const ExtArgs& a, int i, int j, int 
   }
   (AXIS == 0 ? a.ug : (AXIS == 1 ? a.vg : a.wg))[r.off] = ug;
 }
-// 53.3 us at 128^3, 87.8 with a thread per face, six FP64 operations on each and n read everywhere: a face away from the
-// interface takes a subtraction and a multiply-add now.
-static __global__ void __launch_bounds__(kCornerThreads, 2) k_extend_epi(ExtArgs a) {
-  const int i = blockIdx.x * 32 + (threadIdx.x & 31), k = blockIdx.z;
-  for (int q = threadIdx.x >> 5; q < kCornerRows; q += blockDim.x >> 5) {
-    const int j = blockIdx.y * kCornerRows + q;
-    extend_face<0>(a, i, j, k);
-    extend_face<1>(a, i, j, k);
-    extend_face<2>(a, i, j, k);
-  }
+// 39.1 us at 128^3 (87.8 with a thread per face, six FP64 operations on each and n read everywhere): a face away from the
+// interface takes a subtraction and a multiply-add; 126 us at 256 x 256 x 128, 334 before.
+static __global__ void __launch_bounds__(kCornerThreads) k_extend_epi(ExtArgs a) {
+  int i, j, axes;
+  const int k = flat_corner(a.g, i, j, axes);
+  if (axes & 1) extend_face<0>(a, i, j, k);
+  if (axes & 2) extend_face<1>(a, i, j, k);
+  if (axes & 4) extend_face<2>(a, i, j, k);
 }
 
 // Variable-density pressure splitting (§3.2, Eq. lap_p and the update after it): u* -= dt (1/rho_f - 1/rho0)
@@ -345,17 +382,12 @@ __device__ __forceinline__ void vd_face(const VdArgs& a, int i, int j, int k) {
   double* F = AXIS == 0 ? a.u : (AXIS == 1 ? a.v : a.w);
   F[r.off] = fma(-(h * one_path(c)), d, F[r.off]);
 }
-// (Lanes run over the corners of a plane row after row: a tile of 32 a row leaves lanes of the FP64 pipe's turns idle where a
-// row is no multiple of 32: 128^3 86 -> 74 us, 20 x 20 x 160 25 -> 14, 34 x 134 x 64 58 -> 30.)
-constexpr int kVdThreads = 128;
-inline dim3 vd_grid(const GridDev& g) {
-  return dim3((unsigned)((nface(g.nx, g.bcx) * nface(g.ny, g.bcy) + kVdThreads - 1) / kVdThreads), (unsigned)nface(g.nz, g.bcz));
-}
-static __global__ void __launch_bounds__(kVdThreads) k_vd_predict(VdArgs a) {
-  const int c = blockIdx.x * kVdThreads + threadIdx.x, fx = nface(a.g.nx, a.g.bcx), j = c / fx, i = c - j * fx, k = blockIdx.y;
-  vd_face<0>(a, i, j, k);
-  vd_face<1>(a, i, j, k);
-  vd_face<2>(a, i, j, k);
+static __global__ void __launch_bounds__(kCornerThreads) k_vd_predict(VdArgs a) {
+  int i, j, axes;
+  const int k = flat_corner(a.g, i, j, axes);
+  if (axes & 1) vd_face<0>(a, i, j, k);
+  if (axes & 2) vd_face<1>(a, i, j, k);
+  if (axes & 4) vd_face<2>(a, i, j, k);
 }
 
 }  // namespace vofp

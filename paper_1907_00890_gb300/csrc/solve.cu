@@ -379,9 +379,10 @@ static int project_common(vofp_plan* pl, int mode, XArgs& xa, double* u, double*
     if (s) return s;
   }
   const GridDev g = grid_dev(pl);
+  const bool flat = corner_flat(g);
   VOFP_LAUNCH(KID_GRAD, st,
-              k_grad_update<<<corner_grid(g), corner_threads(g), 0, st>>>(g, pout, u, v, w, dt_over_rho0, dt_over_rho0 * g.rdx,
-                                                                      dt_over_rho0 * g.rdy));
+              ((flat ? k_grad_update<true> : k_grad_update<false>)<<<flat ? flat_grid(g) : corner_grid(g), kCornerThreads, 0, st>>>(
+                  g, pout, u, v, w, dt_over_rho0, dt_over_rho0 * g.rdx, dt_over_rho0 * g.rdy)));
   const int ls = cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
   if (pl->opts.prec != VOFP_FP64) {
     if (ls) return ls;
@@ -432,7 +433,7 @@ static int extend_common(vofp_plan* pl, const double* u, const double* v, const 
   ea.ug = ug;
   ea.vg = vg;
   ea.wg = wg;
-  VOFP_LAUNCH(KID_EXTEND_EPI, st, k_extend_epi<<<corner_grid(ea.g), corner_threads(ea.g), 0, st>>>(ea));
+  VOFP_LAUNCH(KID_EXTEND_EPI, st, k_extend_epi<<<flat_grid(ea.g), kCornerThreads, 0, st>>>(ea));
   const int ls = cudaGetLastError() == cudaSuccess ? VOFP_OK : VOFP_ERR_CUDA;
   if (pl->opts.prec != VOFP_FP64) {
     if (ls) return ls;
@@ -505,7 +506,7 @@ extern "C" int vofp_project_vd(vofp_plan* pl, double* u, double* v, double* w, c
   va.u = u;
   va.v = v;
   va.w = w;
-  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<vd_grid(va.g), kVdThreads, 0, st>>>(va));
+  VOFP_LAUNCH(KID_VD, st, k_vd_predict<<<flat_grid(va.g), kCornerThreads, 0, st>>>(va));
   if (cudaGetLastError() != cudaSuccess) return VOFP_ERR_CUDA;
   return vofp_project(pl, u, v, w, src, dt / rho0, p, stream, info);
 }
