@@ -990,8 +990,10 @@ def measured_traffic(workload, kernel):
 def algorithmic(kname, n):
     """Algorithmic HBM bytes and FP64 flops of one launch of kernel class ``kname`` on an n-grid.
 
-    Bytes: each compulsory array read or written once (8 B per FP64 value).  Flops: the transforms count none (they run
-    in 64-bit fixed point on the integer pipe; only right-hand sides are formed in FP64); the z recurrence with
+    Bytes: each compulsory array read or written once (8 B per FP64 value).  Flops: the transforms count none on the FP64
+    unit, only right-hand sides do: the grids reported here (128^3, 512^3, the ensembles) transform in 64-bit fixed
+    point on the integer pipe, in FP32 or in FP32 pairs.  (An FP64 plan of another size whose axes keep FP64 butterflies,
+    see ``fx_takes`` in csrc/fxfft.cuh, does some 2.5 log2 m a value more than is counted.)  The z recurrence with
     plan-time factors 6 per point (forward multiply-add and multiply, back multiply-add, output scale);
     stencils their adds and multiplies (a multiply-add counts 2): the velocity correction a difference and a
     multiply-add per face (3, one more product on z faces: 10 per cell), the extension a difference, two face

@@ -107,7 +107,8 @@ int fp64_solve(vofp_plan* pl, int mode, XArgs xa, double* pout, cudaStream_t st,
 struct YArgs;
 bool ypass_tma_f64(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st);
 // The fixed-point transform passes of FP64 (T = double) and FP32-pair (T = ff) spectra (fxpass.cuh, instantiated in
-// fx64.cu and fxff.cu); false: the axis' length has none (a Bluestein length, a plan without the tables), not run.
+// fx64.cu and fxff.cu); false: the axis has no tables (longer than 2048, a prime above the limits, a length that would lose
+// accuracy or a grid on which floating point is faster: see fx_takes), not run.
 template <typename T>
 void init_fx_attributes();
 template <typename T>
