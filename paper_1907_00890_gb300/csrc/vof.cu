@@ -29,9 +29,10 @@ namespace vofp {
 // final_corr_2 for plane m - 1, which needs C** of m - 2, m - 1 and m.  C^n, uG, vG, wG are read and C^{n+1}
 // written once per cell (40 bytes) and C*, C** never leave shared memory; the price is the recomputed halo rows
 // and planes (x step x (1 + 2/kVofTY)(1 + 2/kVofKC), y step x (1 + 2/kVofKC)).  Cells whose neighbours hold the same C -- the
-// inside of each phase -- take no FP64 arithmetic: 128^3 droplet 110 us, 218 when every cell did
+// inside of each phase -- take no FP64 arithmetic: 128^3 droplet 108 us, 218 when every cell did on tiles of 32 x 16 x 16
 // (FP64 pipe 77-84% busy).  Small tiles, for all their halo: the interface makes some tiles long and the others short
-// (32 x 16 x 16 cells 166 us, 16 x 4 126, 8 x 16 131, 4 x 8 125).
+// (32 x 16 x 16 cells 166 us, 16 x 4 126, 8 x 16 131, 4 x 8 125); a C that varies in every cell takes 211 us (214 on the
+// large tiles without the test), 472 at 250 x 150 x 128 (461).
 constexpr int kVofTX = 32, kVofTY = 8, kVofKC = 4;
 
 __device__ __forceinline__ int wrap_clamp(int j, int n, int bc) {

@@ -8,7 +8,7 @@ import pytest
 from paper_1907_00890_gb300 import synth
 
 pytestmark = pytest.mark.gpu
-N, BC = (512, 1, 1024), ("P", "P", "NN")  # one y row: the x spectrum goes straight to the z pass
+N, BC = (512, 1, 1400), ("P", "P", "NN")  # one y row: the x spectrum goes straight to the z pass
 
 
 def solve(f):
