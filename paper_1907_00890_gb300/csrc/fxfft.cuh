@@ -8,8 +8,9 @@
 //
 // Measured (CUDA events, FP64 spectra, P, P, NN; FP64 butterflies -> fixed point): 128^3 divergence + x 92.7 -> 55 us,
 // x 69.5 -> 28.7, y 62.0 / 63.6 -> 20.4 / 23.4, inverse x 65.5 -> 24.8; 320 x 320 x 640 (run-time stages of radix 5, 8, 8)
-// x 2.30 -> 1.28 ms, y 2.09 -> 0.68, inverse x 2.16 -> 0.81.  Bound now by instruction issue (some 130 a value: a third
-// in the two conversions) and the latency of the 64-bit carry chains.
+// x 2.30 -> 1.28 ms, y 2.09 -> 0.68, inverse x 2.16 -> 0.81.  Bound now by the integer pipe, 52 to 57% busy over a whole
+// pass (ncu at 128^3: 143 to 198 instructions a value, issue 38 to 46%), and by the latency of the 64-bit carry chains with a
+// third of the warps that an SM can hold.
 //
 // Scaling.  A complex value z of a line satisfies |z| <= 2^61.5 throughout.  A twiddle product leaves a quarter of
 // its exact value (two factors of 2^62 and the upper 64 bits of the product), a radix-R stage adds up R values, so
@@ -538,7 +539,7 @@ __device__ __forceinline__ long long fx_value(const FxSum& f, int lam) {
 }
 
 // A rolled stage of an odd prime RAD >= 7 from src into dst (see fft_stage_odd); src is scratch afterwards.  Bound by
-// instruction issue, some 50 a product pair: the weights lie in shared memory with their signs, and the lift of a line
+// instruction issue: the weights lie in shared memory with their signs, and the lift of a line
 // with little growth is applied to the sums.
 template <bool TWS>
 __device__ __noinline__ void fx_stage_odd(int so, int dof, int st, int lgB, int n, int Ns, unsigned magic, int RAD, int twoff,
