@@ -158,34 +158,25 @@ inline long fx_tiles8(int nx, int ny, int nz, bool y) {
 // 1.4-2.2 everywhere.  FP32 pairs, x: 0.6-0.95 up to 500,000 cells, 0.81-1.2 at 2,000,000, 0.87-1.16 at 2,400,000, 1.0-1.28 at
 // 2,800,000, 1.1-1.4 at 12,000,000; y: up to 50 samples 1.0-1.28 from 2,400,000, 72 to 100 0.74-1.08 below 6,000,000 and 1.0-1.2 at 8 to 12
 // million, beyond that 0.66-0.98 up to 6,000,000 and 0.87-1.1 at 8 to 12.
-// Lengths with a prime above 13: a rolled stage costs p products a value, the floating-point passes' Bluestein form two
-// transforms of two to three times the length.  FP64: p up to 89 0.9-2.3 below 250,000 cells, 1.3-4.9 above; 97 to 113 on x 0.78-1.35 below
-// 250,000, 1.2-2.6 above; 127 to 199 0.54-1.0 below 500,000, 1.03-2.4 above; y 1.0-6.6.  FP32 pairs: p up to 43 0.86-2.4; 47 and
-// 53 0.76-1.1 from 64,000 to 250,000, 0.92-1.5 above.  Where a one-warp block holds at most 128 values, four a lane, the chain
-// is short enough for any of them: 1.0-1.9.
+// Lengths with a prime above 13 (p to 199; FP32 pairs 53): a rolled stage costs p products a value, the floating-point passes'
+// Bluestein form two transforms of two to three times the length.  FP64: x 0.99-2.3 at 16,000 to 125,000 cells (179: 0.99, 199: 1.11,
+// 127: 1.27), 1.03-4.9 above, y 1.35-6.6; FP32 pairs 1.0-3.  (With an eighth of a tile's values in threads on small grids too: FP64
+// x 0.54-1.0 for p from 127 on below 500,000 cells, FP32 pairs 0.76-1.1 for 47 and 53.  See fx_threads.)
 // `force` (VOFP_FX=1 when the plan is created): fixed point whatever the grid, for comparisons.
 inline bool fx_takes(const FftDesc& fd, bool ff, bool y, int nx, int ny, int nz, bool force) {
   FxDesc fx;
-  int prime = 1;
-  for (int s = 0; s < fd.nst; ++s) {
+  for (int s = 0; s < fd.nst; ++s)
     if (fd.radix[s] > (ff ? 53 : kFxMaxPrime)) return false;
-    if (fd.radix[s] != 8 && fd.radix[s] != 4 && fd.radix[s] > prime) prime = fd.radix[s];
-  }
   if (!fx_desc(fd, &fx)) return false;
   // (stages of radix 3 err more in FP64 too; a Bluestein form by 4e-16 to 7e-16)
   if (!fd.bm && !ff && fx_noise(fd) > (fx.two ? 1.45e-16 : 2e-16)) return false;
-  if (force) return true;
+  if (force || fd.bm) return true;
   const long cells = (long)nx * ny * nz;
-  const int n = fd.n, lgB = fx_lgB(n, fx_tiles8(nx, ny, nz, y), y ? 1 : 0);
-  if (fd.bm) {
-    if ((n << lgB) <= 128) return true;
-    if (ff) return prime <= 43 || cells >= 500000;
-    return y || prime <= 89 || cells >= (prime <= 113 ? 250000 : 500000);
-  }
+  const int n = fd.n;
   const bool pow2 = (n & (n - 1)) == 0;
   if (pow2 && n >= 32 && n <= 512) {
     if (ff) return cells >= (n <= 64 ? 480000 : 700000);
-    return n >= 64 || lgB == fx_ct_lgB(5) || cells >= 480000;
+    return n >= 64 || cells >= 480000 || fx_lgB(n, fx_tiles8(nx, ny, nz, y), y ? 1 : 0) == fx_ct_lgB(5);
   }
   if (ff) {
     if (y) return cells >= 2400000 && (n <= 50 || (n <= 100 && cells >= 8000000));
@@ -779,6 +770,15 @@ __device__ __forceinline__ cfx fx_down(cfx v, int rho) {
 
 // Threads for a tile of 2^lgB lines of n: an eighth of its values, whole warps.
 inline int fx_threads(int n, int lgB) { return (((n << lgB) + 7) / 8 + 31) / 32 * 32; }
+// The same for `blocks` tiles: where they leave an SM less than half its warps, a length with a rolled stage takes more of them, down to
+// a value a thread: the stage's items, p products each, are what such a pass waits for (x pass of 199 x 199 x 3 72 us with an eighth,
+// 33 so).
+inline int fx_threads(const FxDesc& fd, int lgB, long blocks) {
+  int th = fx_threads(fd.n, lgB);
+  if (fd.two)
+    while (2 * th <= 256 && 2 * th < (fd.n << lgB) + 32 && blocks * (2 * th / 32) <= 152 * 32) th *= 2;
+  return th;
+}
 constexpr int kFxMaxThreads = 256;  // (of the run-time lengths)
 // Launch bounds.  The compiled-in lengths are held to 72 registers a thread (seven blocks of 128 threads an SM): more
 // warps hide more of the integer carry chains' latency than the registers would save (y pass of 128^3: 25.0 us at 96

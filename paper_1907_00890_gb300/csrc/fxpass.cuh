@@ -117,7 +117,7 @@ bool fx_xfwd(vofp_plan* pl, int mode, const XArgs& xa, cudaStream_t st) {
   const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
   int lgn;
   if (!fx_tables<T>(pl, 0, 0, mode == RHS_DIV_STEFAN, &f, &lgn)) return false;
-  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
+  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd, f.lgB, grid);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
   const int kid = mode == RHS_F ? KID_XFWD : (mode == RHS_DIV ? KID_XFWD_DIV : (mode == RHS_RESID ? KID_RESID : KID_XFWD_DIVSTEF));
   const FxXFwd kern = mode == RHS_STEFAN ? nullptr : fx_xfwd_kernel<T>(mode, lgn);
@@ -132,7 +132,7 @@ bool fx_ypass(vofp_plan* pl, const YArgs& ya, bool inv, cudaStream_t st) {
   const int nx = pl->n[0], nz = pl->n[2];
   if (!fx_tables<T>(pl, 1, 1, false, &f, &lgn)) return false;
   const dim3 grid((nx + (2 << f.lgB) - 1) / (2 << f.lgB), nz);
-  const int th = fx_threads(f.fd.n, f.lgB);
+  const int th = fx_threads(f.fd, f.lgB, (long)grid.x * nz);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
   VOFP_LAUNCH(inv ? KID_YINV : KID_YFWD, st, (fx_ypass_kernel<T>(inv, lgn)<<<grid, th, sm, st>>>(ya, f)));
   return true;
@@ -143,7 +143,7 @@ bool fx_xinv(vofp_plan* pl, const XInvArgs& xi, cudaStream_t st) {
   const long npairs = ((long)pl->n[1] * pl->n[2] + 1) / 2;
   int lgn;
   if (!fx_tables<T>(pl, 0, 0, false, &f, &lgn)) return false;
-  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd.n, f.lgB);
+  const int grid = (int)((npairs + (1 << f.lgB) - 1) >> f.lgB), th = fx_threads(f.fd, f.lgB, grid);
   const size_t sm = fx_smem(f.fd, f.lgB, f.st);
   const FxXInv kern = fx_xinv_kernel<T>(lgn, xi.p && !xi.accumulate && !xi.mean_out && !xi.d2_out);
   if (!kern) return false;

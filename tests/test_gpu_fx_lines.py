@@ -1,6 +1,6 @@
 """Both sides of the lines at which a plan takes its x and y transforms in fixed point: grids of one-warp tiles of 32 samples, three
-short stages, primes above 89, FP32 pairs of powers of two, of other lengths and of primes above 43, against the CPU
-oracle at the parity bars."""
+short stages, FP32 pairs of powers of two and of other lengths; and grids of prime lengths whose tiles take an eighth of
+their values in threads, or more, against the CPU oracle at the parity bars."""
 import numpy as np
 import pytest
 
